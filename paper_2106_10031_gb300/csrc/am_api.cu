@@ -611,6 +611,8 @@ am_status am_load_mlp(am_ctx *ctx, const am_mlp_desc *dsc, int *net_id)
     nd.w_out_hi = nh.fblob + offW;
     nd.w_out_lo = nh.fblob + lo_off + offW;
     nd.b_out = dsc->b_out;
+    nd.b_out_hi = (float)dsc->b_out;
+    nd.b_out_lo = (float)(dsc->b_out - (double)nd.b_out_hi);
     nd.M = M;
     nd.n_units = n_units;
     nd.w_heads = M ? nh.blob + offH : nullptr;

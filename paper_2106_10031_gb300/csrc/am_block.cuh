@@ -96,6 +96,13 @@ __device__ __forceinline__ unsigned long long child_word(unsigned long long x, i
     return x;
 }
 
+// the words of two keys a and b crossed at fa and fb, compared (max-pooled nets; out of line)
+static __device__ __noinline__ unsigned long long pooled_diff(unsigned long long a, unsigned long long b, int w, unsigned fa,
+                                                       unsigned fb, int pool0, int pool1)
+{
+    return child_word(a, w, fa, pool0, pool1) ^ child_word(b, w, fb, pool0, pool1);
+}
+
 // key(pa) crossed at fa == key(pb) crossed at fb ?  (kNoFlip = nothing crossed)
 // Keys written by other blocks of a running kernel are read through L2 (ld.global.cg): the
 // SM's L1 is not coherent with other SMs' writes and may hold a stale copy of the line.
@@ -112,51 +119,88 @@ __device__ __forceinline__ bool ref_keys_equal(const Arena &ar, int64_t pa, unsi
 }
 
 // Alg. 1 steps 10-11: the neighbour across plane `flip` (hash h) is pushed unless it was seen
-// before.  The slot records (parent, flip), from which any later probe rebuilds the key, so a
-// claim never waits for a key to be written.  A claim hands out the next cell id, writes the
-// new cell's record there (key, net, hash, the crossed plane as the new cell names it, entry,
-// or flip when entry < 0, and a point of the shared edge), then publishes it through ready[id].
-// pool0, pool1: the pooling bits of a max-pooled net (child_word).
-__device__ __forceinline__ void insert_neighbor(const Arena &ar, const unsigned *mask, int64_t parent, int net,
-                                                unsigned flip, unsigned long long h, float px, float py, float pz,
-                                                int pool0 = kNoPool, int pool1 = kNoPool, int entry = -1)
+// before; a whole warp calls this, one neighbour per lane with `on` set.  The slot records
+// (parent, flip), from which any later probe rebuilds the key, so a claim never waits for a key
+// to be written.  The lanes that claimed a slot take their cell ids from one atomic, write the
+// new cells' records there (key, net, hash, the crossed plane as the new cell names it, entry,
+// or flip when entry < 0, and a point of the shared edge), then publish them through ready[id].
+// pool0, pool1: the pooling bits of a max-pooled net (child_word).  Four words of a compared key
+// are in flight at once.
+__device__ __forceinline__ void insert_neighbors(const Arena &ar, const unsigned *mask, int64_t parent, int net,
+                                                 bool on, unsigned flip, unsigned long long h, float px, float py,
+                                                 float pz, int pool0, int pool1, int entry)
 {
+    const int lane = threadIdx.x & 31;
     const unsigned long long mine = slot_make(h, (unsigned long long)parent, flip);
-    unsigned long long pos = h & ar.slot_mask;
-    for (int probe = 0; probe < kMaxProbe; ++probe) {
-        const unsigned long long cur = atomicCAS(ar.slots + pos, 0ull, mine);
-        if (cur == 0ull) {
-            long long id = (long long)atomicAdd(ar.counters + kNCells, 1ull);
-            if (id >= ar.cap) {
-                atomicOr(ar.counters + kStatus, kStCellCap);
-                return;
+    bool claimed = false;
+    if (on) {
+        unsigned long long pos = h & ar.slot_mask;
+        int probe = 0;
+        for (; probe < kMaxProbe; ++probe) {
+            const unsigned long long cur = atomicCAS(ar.slots + pos, 0ull, mine);
+            if (cur == 0ull) { claimed = true; break; }
+            if (slot_tag(cur) == hash_tag(h)) {
+                // Keys written by other blocks of a running kernel are read through L2 (ld.global.cg):
+                // the SM's L1 is not coherent with other SMs' writes
+                const int64_t pb = slot_parent(cur);
+                const unsigned fb = slot_flip(cur);
+                const int nb = __ldcg(ar.net + pb);
+                unsigned long long diff = 0ull;
+#pragma unroll 1
+                for (int w0 = 0; w0 < ar.kw; w0 += 4) {
+                    unsigned long long kb[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) kb[q] = w0 + q < ar.kw ? __ldcg(ar.keys + pb * ar.kw + w0 + q) : 0ull;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (w0 + q < ar.kw) {
+                            // the parent's key is its state, held by the block in shared memory
+                            const int w = w0 + q;
+                            unsigned long long d = kb[q] ^ ((unsigned long long)mask[2 * w] | ((unsigned long long)mask[2 * w + 1] << 32));
+                            if (pool0 == kNoPool) {      // two unit planes: two bits flip (fb may be kNoFlip: no word)
+                                if ((int)(flip >> 6) == w) d ^= 1ull << (flip & 63);
+                                if ((int)(fb >> 6) == w && fb != kNoFlip) d ^= 1ull << (fb & 63);
+                                diff |= d;
+                            } else {
+                                diff |= pooled_diff(d ^ kb[q], kb[q], w, flip, fb, pool0, pool1);
+                            }
+                        }
+                }
+                if (nb == net && diff == 0ull) break;
             }
-            // the parent's key is its state, held by the block in shared memory
-            unsigned long long *kn = ar.keys + id * ar.kw;
-            for (int w = 0; w < ar.kw; ++w) {
-                const unsigned long long x = (unsigned long long)mask[2 * w] | ((unsigned long long)mask[2 * w + 1] << 32);
-                kn[w] = child_word(x, w, flip, pool0, pool1);
-            }
-            ar.net[id] = net;
-            ar.hash[id] = h;
-            ar.nverts[id] = -1;
-            ar.entry_plane[id] = entry >= 0 ? entry : (int32_t)flip;
-            ar.parent[id] = (int32_t)parent;
-            ar.entry_pt[id * 3 + 0] = px;
-            ar.entry_pt[id * 3 + 1] = py;
-            ar.entry_pt[id * 3 + 2] = pz;
-            // publish: every write above is visible to whoever acquires the flag
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ar.ready + id), "r"(1u) : "memory");
-            return;
+            pos = (pos + 1) & ar.slot_mask;
         }
-        if (slot_tag(cur) == hash_tag(h)) {
-            const int64_t pb = slot_parent(cur);
-            if (__ldcg(ar.net + pb) == net && ref_keys_equal(ar, parent, flip, pb, slot_flip(cur), pool0, pool1))
-                return;
-        }
-        pos = (pos + 1) & ar.slot_mask;
+        if (probe == kMaxProbe) atomicOr(ar.counters + kStatus, kStHashFull);
     }
-    atomicOr(ar.counters + kStatus, kStHashFull);
+    __syncwarp();
+    const unsigned who = __ballot_sync(0xffffffffu, claimed);
+    if (who == 0u) return;
+    const int lead = __ffs(who) - 1;
+    unsigned long long base = 0ull;
+    if (lane == lead) base = atomicAdd(ar.counters + kNCells, (unsigned long long)__popc(who));
+    base = __shfl_sync(0xffffffffu, base, lead);
+    if (!claimed) return;
+    const long long id = (long long)base + __popc(who & ((1u << lane) - 1u));
+    if (id >= ar.cap) {
+        atomicOr(ar.counters + kStatus, kStCellCap);
+        return;
+    }
+    unsigned long long *kn = ar.keys + id * ar.kw;
+#pragma unroll 1
+    for (int w = 0; w < ar.kw; ++w) {
+        const unsigned long long x = (unsigned long long)mask[2 * w] | ((unsigned long long)mask[2 * w + 1] << 32);
+        kn[w] = child_word(x, w, flip, pool0, pool1);
+    }
+    ar.net[id] = net;
+    ar.hash[id] = h;
+    ar.nverts[id] = -1;
+    ar.entry_plane[id] = entry >= 0 ? entry : (int32_t)flip;
+    ar.parent[id] = (int32_t)parent;
+    ar.entry_pt[id * 3 + 0] = px;
+    ar.entry_pt[id * 3 + 1] = py;
+    ar.entry_pt[id * 3 + 2] = pz;
+    // publish: every write above is visible to whoever acquires the flag
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ar.ready + id), "r"(1u) : "memory");
 }
 
 // The same push by a whole warp (every lane calls it with the same arguments): lane 0 claims

@@ -68,6 +68,7 @@ struct NetDev {
     const double *w_out;
     const float *w_out_hi, *w_out_lo;
     double b_out;
+    float b_out_hi, b_out_lo;    // b_out as a double-float pair
     // tensor-core compose: W_l (hidden part) as three BF16 parts (hi, mid, lo) in mma.m16n8k16
     // A-fragment order, tile (mt, kt) at (mt * Kt + kt) * 96 uint4 (32 lanes per part), and the
     // per row m of W_l the pair (|W_m|_2, max_j |W_mj|)

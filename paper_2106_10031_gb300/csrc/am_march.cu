@@ -4,11 +4,12 @@
 //   a2 compose : Z_l = W_l diag(s_{l-1}) Z_{l-1} + C_l (Lemma 1, Cor. 1) over the active
 //                neurons of the previous layer, then a_F (Eq. 8);
 //   a3 rows    : c_k = (1 - 2 s_k) Z_k (Eq. 10) plus the box rows;
-//   a4 clip    : the face plane a_F [x;1] = 0 (Eq. 12) starts as a square around the box
-//                section.  Warp 0 cuts it by the 32 rows nearest to a point known to lie on
-//                the face (the midpoint of the edge the cell was entered through, or the seed
-//                point) in order of distance, each cut re-solving its two new vertices from
-//                their planes (Eq. 11);
+//   a4 clip    : the lines in which the rows nearest to a point known to lie on the face (the
+//                midpoint of the edge the cell was entered through, or the seed point) and the
+//                box's rows meet the face plane a_F [x;1] = 0 (Eq. 12) are cut against each other
+//                all at once, and what is left of them closes into the polygon (fast_face); a
+//                face this does not settle is cut out of a square around the box section by its
+//                32 candidate rows one by one (slow_clip).  Vertices from their planes (Eq. 11);
 //   a5 check   : every thread then tests every row at every vertex of that polygon (Alg. 1
 //                step 8 for the output); a violated row is cut in and the check repeated, so
 //                the result is the clip by all rows whatever the candidates were;
@@ -35,32 +36,55 @@
 
 namespace am {
 
-// Threads per block and the minimum resident blocks per SM the compiler must allow for
-// (register budget); both can be set at build time for launch-shape sweeps.
-#ifndef AM_THREADS
-#define AM_THREADS 256
-#endif
+// The minimum resident blocks per SM the compiler must allow for (register budget); can be set at
+// build time for launch-shape sweeps.
 #ifndef AM_MIN_BLOCKS
 #define AM_MIN_BLOCKS 2
 #endif
-constexpr int kT = AM_THREADS;    // threads per block
+constexpr int kT = 256;           // threads per block
 constexpr int kNW = kT / 32;      // warps per block
 constexpr int kMaxPoly = 64;      // polygon vertices in flight
 constexpr int kNear = 32;         // rows clipped by warp 0 before the full check
 constexpr int kPicks = kNear / kNW;   // candidates each warp contributes
-static_assert(kT % 32 == 0 && kNW <= 32 && kNear % kNW == 0, "block shape");
+constexpr int kLines = 64;        // candidate lines of the one-pass polygon: the box's and the nearest rows'
+constexpr int kParts = kT / kLines;   // threads that share a line's interval
+constexpr int kPartBytes = 40 * kT;   // scratch: the one-pass polygon, the proposal's layers
+constexpr int kLinePicks = 10;    // nearest rows a warp contributes at most (all of them when N <= 32)
+constexpr int kFastFix = 4;       // rounds of the one-pass polygon before the sequential clip takes the cell
+// What a cell's compose reads of its net, kept in shared memory while the block stays on the net: every
+// field of the global record costs an L2 round trip per cell (taking a cell from the queue empties
+// the L1).  The weights lie at offsets of one FP64 block and of its copy as double-float pairs.
+struct NetHot {
+    int id;                       // the net (-1: none)
+    int L, N, units, M, fp64_only, df_ok, ws;   // ws: weights (FP64 words from C_1 to the end of the hidden layers)
+    float b_out_hi, b_out_lo;
+    double b_out;
+    const double *d;              // C_1, FP64
+    const float *h, *l;           // the same as hi and lo words
+    int offA[kMaxLayers + 1], offC[kMaxLayers + 1], offw;
+    short width[kMaxLayers + 2], row0[kMaxLayers + 2];
+};
+constexpr int kOHot = 9 * kT * 4;   // its place in the scratch region: past the proposal's layers
+
+static_assert(2 * ((kMaxNeurons + 63) / 64) <= kT, "one thread per 32-bit word of a key");
+static_assert(kT % 32 == 0 && kNW <= 32 && kNear % kNW == 0 && kT >= kLines, "block shape");
+static_assert(kParts == 4 && 256 + 16 * kLines * 2 + 16 * kLines <= 3328 && 3328 + 32 * 8 <= kOHot && kOHot + sizeof(NetHot) <= kPartBytes,
+              "the scratch region");
 constexpr int kMaxFix = 8;        // check / fix-up rounds
 constexpr int kThreadPushWords = 8;   // keys up to this many 64-bit words are pushed by one thread per edge
 constexpr float kU = 5.9604645e-8f;            // 2^-24
+constexpr float kTiny = 1e-30f, kHuge = 1e30f;   // |normal|^2 outside of which FP32 does not judge a row
 constexpr float kDfLoose = 1e-6f;              // certified row error (as a distance) beyond which kDF gives up
 constexpr double kVertexTol = 1e-5;            // largest vertex error bound (relative) kept from kDF
 
 enum { kFP64 = 0, kDF = 1 };
 
 // Optional per-phase cycle counters (build with -DAM_PHASE_TIMERS): thread 0 of each block adds
-// the clock64() cycles of each phase of each cell to counters[kPhase0 + phase * kCtrStride].
+// the clock64() cycles of each phase of each cell to counters[kPhase0 + phase * kCtrStride].  Every
+// thread reads the clock: a read by one thread splits its warp, and what it then costs to run the code
+// after it twice was most of what the timers showed.
 #ifdef AM_PHASE_TIMERS
-#define AM_TICK(t) do { if (threadIdx.x == 0) (t) = clock64(); } while (0)
+#define AM_TICK(t) do { (t) = clock64(); } while (0)
 #define AM_PHASE(a, i, t0, t1) do { if (threadIdx.x == 0) atomicAdd((a).ar.counters + kPhase0 + (i) * kCtrStride, \
     (unsigned long long)((t1) - (t0))); } while (0)
 #else
@@ -71,40 +95,36 @@ enum { kFP64 = 0, kDF = 1 };
 // ------------------------------------------------------------------------------------------
 // shared-memory layout
 
-struct Lay {
-    int mask, rows, err, rinv, carry, act, part, pv, pe, pf, vf, dvb, near, viol, sc, total;
-};
+// The regions of fixed size come first, at constant offsets; then the key and the rows' arrays,
+// sized by the largest loadable net.
+constexpr int al16(int x) { return (x + 15) & ~15; }
+constexpr int kOSc = 0;                                     // scalars
+constexpr int kONear = kOSc + 512;
+constexpr int kOPe = kONear + 4 * 4 * kNear;
+constexpr int kODvb = kOPe + 2 * kMaxPoly * 4;
+constexpr int kOVf = kODvb + kMaxPoly * 4;
+constexpr int kOPf = kOVf + kMaxPoly * 4 * 4;
+constexpr int kOPv = kOPf + 2 * kMaxPoly * 3 * 4;
+constexpr int kOPart = kOPv + 2 * kMaxPoly * 3 * 8;
+constexpr int kOMask = kOPart + kPartBytes;
+static_assert(kONear % 16 == 0 && kOVf % 16 == 0 && kOPv % 16 == 0 && kOPart % 16 == 0 && kOMask % 16 == 0, "alignment");
 
-__host__ __device__ inline int al16(int x) { return (x + 15) & ~15; }
-
-__host__ __device__ inline Lay march_layout(int max_n, int max_w)
+__host__ __device__ inline int lay_rows(int max_n) { return kOMask + al16(((max_n + 63) / 64) * 8); }   // whole key words
+__host__ __device__ inline int lay_nr(int max_n) { return max_n + kBoxPlanes + kSquarePlanes; }
+// rows (32 B each: FP64, or the FP32 hi words, then the lo words), then err, rinv and viol
+__host__ __device__ inline int lay_total(int max_n)
 {
-    Lay s;
-    const int nr = max_n + kBoxPlanes + kSquarePlanes;
-    int o = 0;
-    s.mask = o;  o = al16(o + ((max_n + 63) / 64) * 8);   // the whole key (kw 64-bit words)
-    s.rows = o;  o = al16(o + nr * 32);                 // double[4] (FP64) or float[4] hi + float[4] lo (DF)
-    s.err = o;   o = al16(o + nr * 4);
-    s.rinv = o;  o = al16(o + nr * 4);
-    s.carry = o; o = al16(o + max_w * 4);
-    s.act = o;   o = al16(o + max_w * 4);
-    s.part = o;  o = al16(o + kT * 40);
-    s.pv = o;    o = al16(o + 2 * kMaxPoly * 3 * 8);
-    s.pe = o;    o = al16(o + 2 * kMaxPoly * 4);
-    s.pf = o;    o = al16(o + 2 * kMaxPoly * 3 * 4);
-    s.vf = o;    o = al16(o + kMaxPoly * 4 * 4);
-    s.dvb = o;   o = al16(o + kMaxPoly * 4);
-    s.near = o;  o = al16(o + 2 * kNear * 4 + 2 * kNear * 4);
-    s.viol = o;  o = al16(o + nr * 4);
-    s.sc = o;    o = al16(o + 512);
-    s.total = o;
-    return s;
+    return lay_rows(max_n) + lay_nr(max_n) * 32 + 3 * al16(lay_nr(max_n) * 4);
 }
 
-int march_smem_bytes(int max_n, int max_w) { return march_layout(max_n, max_w).total; }
+int march_smem_bytes(int max_n, int max_w)
+{
+    (void)max_w;
+    return lay_total(max_n);
+}
 
 // The proposal's scores use the compose scratch: 64 features + 2 hidden layers + 2 kT partials.
-int proposal_max_hidden() { return (kT * 10 - 64 - 2 * kT) / 2; }
+int proposal_max_hidden() { return (kOHot / 4 - 64 - 2 * kT) / 2; }
 
 // The tensor-core compose keeps one layer's B fragments (16 bytes per lane per 16 input rows)
 // in the low-part row array (16 bytes per row): 32 ceil(n_{l-1} / 16) <= max_n + 10 rows.
@@ -116,11 +136,18 @@ bool tc_fits(const int *width, int L, int max_n)
 }
 
 struct Sh {
+    NetHot *hot;
+    unsigned long long *zb;       // hash words of the ring's planes
     unsigned *mask;
     double *r64;            // FP64 rows [nr][4]
     float *rhi, *rlo;       // DF rows [nr][4] each
-    float *err, *rinv, *carry;
-    int *act;
+    float *err, *rinv;
+    int *lst;               // the active units, ascending (the violator array, free during the compose)
+    int *lst0;              // lst0[l]: first entry of lst of a unit of layer l (1 .. L), lst0[L + 1] = all
+    float *carry;           // kDF compose: e_j + g |row_j|_1 of every row (the rinv array, free until the compose ends)
+    float4 *line;           // the face's candidate lines (a, b, c, row id) in the face plane's coordinates
+    float4 *seg;            // each line's interval (t0, t1, j0, j1)
+    int *ring;              // 4 x kLines ints of the ring's assembly
     float *partf;
     double *partd;
     double (*pv)[kMaxPoly][3];
@@ -138,37 +165,51 @@ struct Sh {
     int *si;                // 32 ints: 0 m, 1 buf, 2 status, 3 nviol, 4 amb, 5 ndeg, 6 emit, 7 ticket,
                             //          8 near count, 9 fix rounds, 10 a vertex too uncertain
     int *wsum;              // 32 ints
+    float *ent;             // the point the cell was entered through
+    unsigned long long *hsh;   // the cell's hash
+    int *nid;               // and its net
     unsigned long long *blk;   // per-block statistics, flushed once when the block exits:
                                // 0 solved, 1 empty, 2 degenerate, 3 fixups, 4 refined, 5 close calls,
                                // 6 cuts
 };
 
-__device__ inline Sh make_sh(unsigned char *base, int max_n, int max_w)
+extern __shared__ __align__(16) unsigned char march_smem[];
+
+// Every function that is not inlined makes its own view: the pointers are then known to lie in shared
+// memory, most of them at constant offsets (a view passed by reference lives in local memory, and each
+// access through it loads its pointer from there first).
+__device__ __forceinline__ Sh make_sh(int max_n)
 {
-    const Lay L = march_layout(max_n, max_w);
-    const int nr = max_n + kBoxPlanes + kSquarePlanes;
+    unsigned char *const base = march_smem;
+    const int nr = lay_nr(max_n), o = lay_rows(max_n), n4 = al16(nr * 4);
     Sh s;
-    s.mask = (unsigned *)(base + L.mask);
-    s.r64 = (double *)(base + L.rows);
-    s.rhi = (float *)(base + L.rows);
+    s.mask = (unsigned *)(base + kOMask);
+    s.hot = (NetHot *)(base + kOPart + kOHot);
+    s.zb = (unsigned long long *)(base + kOPart + 3328);
+    s.r64 = (double *)(base + o);
+    s.rhi = (float *)(base + o);
     s.rlo = s.rhi + 4 * nr;
-    s.err = (float *)(base + L.err);
-    s.rinv = (float *)(base + L.rinv);
-    s.carry = (float *)(base + L.carry);
-    s.act = (int *)(base + L.act);
-    s.partf = (float *)(base + L.part);
-    s.partd = (double *)(base + L.part);
-    s.pv = (double(*)[kMaxPoly][3])(base + L.pv);
-    s.pe = (int(*)[kMaxPoly])(base + L.pe);
-    s.pf = (float(*)[kMaxPoly][3])(base + L.pf);
-    s.vf = (float(*)[4])(base + L.vf);
-    s.dvb = (float *)(base + L.dvb);
-    s.near_k = (int *)(base + L.near);
+    s.err = (float *)(base + o + 32 * nr);
+    s.rinv = (float *)(base + o + 32 * nr + n4);
+    s.carry = s.rinv;
+    s.viol = (int *)(base + o + 32 * nr + 2 * n4);
+    s.lst = s.viol;
+    s.lst0 = (int *)(base + kOPart);                    // 256 B, then the fast face's scratch
+    s.line = (float4 *)(base + kOPart + 256);
+    s.seg = s.line + kLines;
+    s.ring = (int *)(s.seg + kLines);
+    s.partf = (float *)(base + kOPart);
+    s.partd = (double *)(base + kOPart);
+    s.pv = (double(*)[kMaxPoly][3])(base + kOPv);
+    s.pe = (int(*)[kMaxPoly])(base + kOPe);
+    s.pf = (float(*)[kMaxPoly][3])(base + kOPf);
+    s.vf = (float(*)[4])(base + kOVf);
+    s.dvb = (float *)(base + kODvb);
+    s.near_k = (int *)(base + kONear);
     s.near_d = (float *)(s.near_k + kNear);
     s.near_w = (int *)(s.near_d + kNear);
     s.near_dw = (float *)(s.near_w + kNear);
-    s.viol = (int *)(base + L.viol);
-    double *sc = (double *)(base + L.sc);
+    double *sc = (double *)(base + kOSc);
     s.aF = sc;                                   // 4 doubles
     s.aFhi = (float *)(sc + 4);                  // 4 floats
     s.aFlo = s.aFhi + 4;                         // 4 floats
@@ -176,6 +217,9 @@ __device__ inline Sh make_sh(unsigned char *base, int max_n, int max_w)
     s.si = (int *)(s.eF + 4);                    // 32 ints
     s.wsum = s.si + 32;                          // 32 ints
     s.blk = (unsigned long long *)(s.wsum + 32); // 8 x u64
+    s.hsh = s.blk + 8;
+    s.ent = (float *)(s.hsh + 1);                // 3 floats
+    s.nid = (int *)(s.ent + 3);
     return s;
 }
 
@@ -264,8 +308,9 @@ constexpr int kTcTiles = 4;         // 16-row output tiles a warp accumulates at
 // (random-sign model of the accumulation over T MMAs, each product's share bounded through
 // max|W_mj| and the column norm; the previous rows' estimates propagate by root mean square,
 // without a new factor, so the safety does not compound with depth).
-__device__ __noinline__ void compose_tc_layers(const NetDev &net, const Sh &s, int nr)
+__device__ __noinline__ void compose_tc_layers(const NetDev &net, int max_n, int nr)
 {
+    const Sh s = make_sh(max_n);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t4 = lane & 3;
     uint4 *Bf = reinterpret_cast<uint4 *>(s.rlo);   // per (kt, lane): B1 (x, y), B2 (z, w)
     float *red = reinterpret_cast<float *>(s.wsum);   // 0..3: sum z_c^2, 4: sum e^2 (no scans here)
@@ -373,295 +418,501 @@ __device__ __noinline__ void compose_tc_layers(const NetDev &net, const Sh &s, i
 // ------------------------------------------------------------------------------------------
 // a2/a3: compose the rows of every neuron of the cell, and a_F
 
-// The residual shortcut of layer l (Sec. 5.1) for its row k, FP64: a += sum_j S_kj H_src[j] with
+// The block's copy of a net's record; the caller has a barrier on both sides.
+__device__ __noinline__ void fill_hot(const NetDev *netp, int id, int max_n)
+{
+    const Sh s = make_sh(max_n);
+    NetHot &h = *s.hot;
+    const NetDev &net = *netp;
+    const int l = threadIdx.x, L = net.L;
+    if (l >= 1 && l <= L) {
+        h.width[l] = (short)net.width[l];
+        h.row0[l] = (short)net.row0[l];
+        h.offA[l] = l > 1 ? (int)(net.AT[l] - net.Cl[1]) : 0;
+        h.offC[l] = (int)(net.Cl[l] - net.Cl[1]);
+    }
+    if (l == 0) {
+        h.id = id;
+        h.L = L;
+        h.N = net.N;
+        h.M = net.M;
+        h.units = net.M >= 2 ? net.n_units : net.N;
+        h.fp64_only = net.fp64_only;
+        h.df_ok = net.df_ok;
+        h.b_out = net.b_out;
+        h.b_out_hi = net.b_out_hi;
+        h.b_out_lo = net.b_out_lo;
+        h.d = net.Cl[1];
+        h.h = net.Clhi[1];
+        h.l = net.Cllo[1];
+        h.offw = (int)(net.w_out - net.Cl[1]);
+        h.ws = h.offw + net.width[L];
+    }
+}
+
+// Start the net's weights on their way into the L1 (emptied when the cell was taken), one line per thread,
+// while the cell's record is read; nets too large for the L1 load theirs as they go.
+template <int M>
+__device__ __forceinline__ void touch_weights(const NetHot &h)
+{
+    constexpr int kLine = 128, kMost = 96 * 1024;
+    const int bytes = h.ws * (M == kFP64 ? 8 : 4);
+    if (bytes > (M == kFP64 ? kMost : kMost / 2)) return;
+    unsigned v;
+#pragma unroll 1
+    for (int i = threadIdx.x * kLine; i < bytes; i += kT * kLine) {
+        if (M == kFP64) {
+            asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<const char *>(h.d) + i));
+        } else {
+            asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<const char *>(h.h) + i));
+            asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<const char *>(h.l) + i));
+        }
+    }
+}
+
+// -x by the sign bit: this part's FP64 pipe issues a warp instruction in about 64 cycles
+__device__ __forceinline__ double flip(double x, bool f)
+{
+    return __longlong_as_double(__double_as_longlong(x) ^ (f ? (long long)0x8000000000000000ull : 0ll));
+}
+
+// The residual shortcut of layer l (Sec. 5.1) for column c of its row k, FP64: sum_j S_kj H_src[j] with
 // H_src = diag(g) Z_src (g = 1 on active units, the slope on the others) and the stored row
 // (1 - 2 s) Z, so H_src[j] = -row_j when unit j is active and slope * row_j otherwise; S = null
 // is the identity (H_src[k]).
-__device__ __forceinline__ void add_shortcut(const NetDev &net, const Sh &s, int l, int k, double &a0, double &a1,
-                                             double &a2, double &a3)
+__device__ __forceinline__ double add_shortcut(const NetDev &net, const Sh &s, int l, int k, int c, double a)
 {
     const int src = net.sc_src[l];
-    if (src <= 0) return;
+    if (src <= 0) return a;
     const int rs = net.row0[src], ns = net.width[src];
     const double *S = net.sc_S[l];
     const int j0 = S ? 0 : k, j1 = S ? ns : k + 1;
+#pragma unroll 1
     for (int j = j0; j < j1; ++j) {
         const double w = S ? __ldg(S + (size_t)k * ns + j) : 1.0;
         const int r = rs + j;
         const double f = w * (bit_of(s.mask, r) ? -1.0 : net.slope);
         if (f == 0.0) continue;
-        const double *z = s.r64 + 4 * r;
-        a0 += f * z[0]; a1 += f * z[1]; a2 += f * z[2]; a3 += f * z[3];
+        a += f * s.r64[4 * r + c];
+    }
+    return a;
+}
+
+// The cell's active units in one ascending list (diag(s_l) selects these rows of every layer), with
+// the first entry of each layer: every warp scans the mask's words itself (a popcount scan over
+// its lanes) and writes the entries of the words it owns, so the whole list takes one barrier,
+// the caller's.
+__device__ __forceinline__ void active_list(const NetHot &net, const Sh &s)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu, below = (1u << lane) - 1u;
+    const int units = net.units, nw = (units + 31) >> 5, L = net.L;
+    int base = 0;
+#pragma unroll 1
+    for (int c = 0; c < nw; c += 32) {
+        unsigned word = c + lane < nw ? s.mask[c + lane] : 0u;
+        if (c + lane == units >> 5) word &= (1u << (units & 31)) - 1u;
+        const int n = __popc(word);
+        int inc = n;
+#pragma unroll 1
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(full, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int exc = base + inc - n;
+#pragma unroll 1
+        for (int q = wid; q < 32 && c + q < nw; q += kNW) {
+            const unsigned wq = __shfl_sync(full, word, q);
+            const int eq = __shfl_sync(full, exc, q);
+            if ((wq >> lane) & 1u) s.lst[eq + __popc(wq & below)] = 32 * (c + q) + lane;
+        }
+        if (wid == 0) {
+            const int r0 = lane < L ? net.row0[lane + 1] : 0, w = r0 >> 5;      // L <= 32
+            const int e = __shfl_sync(full, exc, w & 31);
+            const unsigned ww = __shfl_sync(full, word, w & 31);
+            if (lane < L && w >= c && w < c + 32) s.lst0[lane + 1] = e + __popc(ww & ((1u << (r0 & 31)) - 1u));
+        }
+        base += __shfl_sync(full, inc, 31);
+    }
+    if (threadIdx.x == 0) s.lst0[L + 1] = base;
+}
+
+// After the last layer of a max-pooled net
+__device__ __noinline__ void pool_rows(const NetDev &net, int max_n)
+{
+    const Sh s = make_sh(max_n);
+    const int tid = threadIdx.x;
+    // final max pooling (Sec. 5.2): a_F(i) of every head into row n_units + i, then the face
+    // plane a_F(j) of the cell's pooled index j and the pooling rows a_F(i) - a_F(j)
+    const int nL = net.width[net.L], rL = net.row0[net.L];
+    for (int i = 0; i < net.M; ++i) {
+        const double *wh = net.w_heads + (size_t)i * nL;
+        double f[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int k = tid; k < nL; k += kT) {
+            const double w = bit_of(s.mask, rL + k) ? wh[k] : -net.slope * wh[k];
+            if (w != 0.0)
+                for (int c = 0; c < 4; ++c) f[c] -= w * s.r64[4 * (rL + k) + c];
+        }
+        for (int c = 0; c < 4; ++c) f[c] = warp_sum(f[c]);
+        if ((tid & 31) == 0)
+            for (int c = 0; c < 4; ++c) s.partd[4 * (tid >> 5) + c] = f[c];
+        __syncthreads();
+        if (tid == 0) {
+            double F[4] = {0.0, 0.0, 0.0, net.b_heads[i]};
+            for (int w = 0; w < kNW; ++w)
+                for (int c = 0; c < 4; ++c) F[c] += s.partd[4 * w + c];
+            for (int c = 0; c < 4; ++c) s.r64[4 * (net.n_units + i) + c] = F[c];
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        int j = 0;
+        for (int i = 0; i < net.M; ++i)
+            if (bit_of(s.mask, net.n_units + i)) { j = i; break; }
+        for (int c = 0; c < 4; ++c) {
+            s.aF[c] = s.r64[4 * (net.n_units + j) + c];
+            s.aFhi[c] = (float)s.aF[c];
+        }
+        s.eF[0] = 0.0f;
+    }
+    __syncthreads();
+    if (tid < net.M)
+        for (int c = 0; c < 4; ++c) s.r64[4 * (net.n_units + tid) + c] -= s.aF[c];
+    __syncthreads();
+}
+
+// sum over the active units t0 .. t1 of the list of -W_kr row_rc (active: z = -row), FP64: one column c of
+// row k.  The next four weights are on their way while four products issue (a warp's four take about
+// 300 cycles, an L2 round trip 300 to 600); the bounds are the same for every thread, so products
+// past the end are skipped, not issued.
+__device__ __forceinline__ double dot_active(const Sh &s, const double *AT, int nl, int rp, int k, int c, int t0, int t1)
+{
+    double acc = 0.0, w[4] = {0.0, 0.0, 0.0, 0.0};
+    AT += k;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (t0 + u < t1) w[u] = __ldg(AT + (s.lst[t0 + u] - rp) * nl);
+#pragma unroll 1
+    for (int t = t0; t < t1; t += 4) {
+        double wn[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (t + 4 + u < t1) wn[u] = __ldg(AT + (s.lst[t + 4 + u] - rp) * nl);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (t + u < t1) acc -= w[u] * s.r64[4 * s.lst[t + u] + c];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = wn[u];
+    }
+    return acc;
+}
+
+// Rows of every layer in FP64, the nets that compose in FP64 only (leaky units, hidden shortcuts, max
+// pooling): one thread per row and column, as compose<kFP64>.  Returns without a barrier after a_F.
+__device__ __noinline__ void compose_general(const NetDev &net, int max_n)
+{
+    const Sh s = make_sh(max_n);
+    const int tid = threadIdx.x;
+    const bool leaky = net.slope != 0.0;
+    active_list(*s.hot, s);
+    for (int i = tid; i < 4 * net.width[1]; i += kT) s.r64[i] = flip(net.Cl[1][i], bit_of(s.mask, i >> 2));
+    __syncthreads();
+    for (int l = 2; l <= net.L; ++l) {
+        const int nl = net.width[l], rp = net.row0[l - 1], rl = net.row0[l], np = net.width[l - 1];
+        const int t0 = s.lst0[l - 1], t1 = s.lst0[l];
+        const double *AT = net.AT[l], *C = net.Cl[l];
+        const double sl = net.slope;
+        for (int item = tid; item < 4 * nl; item += kT) {
+            const int k = item >> 2, c = item & 3;
+            double acc = 0.0;
+            if (leaky) {
+                // every row takes part (diag(s + slope (1 - s))): active: z = -row (weight 1);
+                // inactive: z = +row, weight slope
+#pragma unroll 4
+                for (int j = 0; j < np; ++j) {
+                    double w = __ldg(AT + (size_t)j * nl + k);
+                    if (!bit_of(s.mask, rp + j)) w *= -sl;
+                    acc -= w * s.r64[4 * (rp + j) + c];
+                }
+            } else {
+                acc = dot_active(s, AT, nl, rp, k, c, t0, t1);
+            }
+            acc = add_shortcut(net, s, l, k, c, acc);
+            s.r64[4 * rl + item] = flip(acc + C[item], bit_of(s.mask, rl + k));
+        }
+        __syncthreads();
+    }
+    if (net.M >= 2) {
+        pool_rows(net, max_n);
+        return;
+    }
+    // a_F = w_out^T diag(s_L) Z_L + [0 | b_out] (Cor. 1, Eq. 8): active: row = -Z (weight 1); inactive:
+    // row = +Z, weight slope; warp 0, lane 4 p + c: column c over every 8th unit
+    if (tid < 32) {
+        const int nL = net.width[net.L], rL = net.row0[net.L], c = tid & 3;
+        double f = 0.0;
+        for (int k = tid >> 2; k < nL; k += 8) {
+            const double w = bit_of(s.mask, rL + k) ? net.w_out[k] : -net.slope * net.w_out[k];
+            if (w != 0.0) f -= w * s.r64[4 * (rL + k) + c];
+        }
+        for (int o = 4; o < 32; o <<= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        if (c == 3) f += net.b_out;
+        if (tid < 4) {
+            s.aF[c] = f;
+            s.aFhi[c] = (float)f;
+        }
+        if (tid == 0) s.eF[0] = 0.0f;
     }
 }
 
-template <int M>
-__device__ __forceinline__ void compose(const NetDev &net, const Sh &s, bool tc, int nrows)
+// kDF: the lanes that share a row's sum, log2.  Layers of at most kNarrow units take one lane per row and
+// column (4 n_l S <= kT), wider ones a lane per row (n_l S <= kT, or S = 1 in several passes).
+constexpr int kNarrow = kT / 8;
+__device__ __forceinline__ int df_split(int nl)
 {
+    return nl <= 8 ? 3 : nl <= 16 ? 2 : nl <= kNarrow ? 1 : nl <= kT / 4 ? 2 : nl <= kT / 2 ? 1 : 0;
+}
+
+// Rows of every layer.  FP64: one thread per row and column (k, c), the four columns of a row in
+// neighbouring lanes, so a layer of n rows issues 4 n / 32 chains of its active units and nothing
+// else on the FP64 pipe, whose warp instructions take about 64 cycles each whatever the lanes do
+// (splitting a narrow layer's sums over the block's warps issued the partial sums' additions on top: a
+// 3-12-6-3-2-1 net's compose took 91,700 cycles so, 7,100 now; 1000 patterns of a 3-[44]x5-1 net
+// 136 us, 98 now).  Double-float: df_split.  One barrier per layer.  Returns without a barrier after
+// a_F, which warp 0 computes.  Two blocks of a 3-[64]x4-1 net keep the FP64 pipe busy through it:
+// 24,600 products per cell at the 1.7 the pipe takes per cycle are 14,500 cycles.
+template <int M>
+__device__ __forceinline__ void compose(const NetDev &netg, const Sh &s, bool tc, int max_n)
+{
+    const NetHot &net = *s.hot;
+    const int nrows = lay_nr(max_n);
     const int tid = threadIdx.x;
+    const unsigned full = 0xffffffffu;
+    if (M == kFP64 && net.fp64_only) {
+        compose_general(netg, max_n);
+        return;
+    }
+    active_list(net, s);
     // layer 1: Z_1 = C_1 (cell independent)
     {
         const int n1 = net.width[1];
-        for (int k = tid; k < n1; k += kT) {
-            const bool act = bit_of(s.mask, k);
-            if (M == kFP64) {
-                const double sg = act ? -1.0 : 1.0;
-                for (int c = 0; c < 4; ++c) s.r64[4 * k + c] = sg * net.Cl[1][4 * k + c];
-            } else {
-                const float sg = act ? -1.0f : 1.0f;
-                float l1 = 0.0f;
-                for (int c = 0; c < 4; ++c) {
-                    const float h = net.Clhi[1][4 * k + c], l = net.Cllo[1][4 * k + c];
-                    s.rhi[4 * k + c] = sg * h;
-                    s.rlo[4 * k + c] = sg * l;
-                    l1 += fabsf(h);
+        if (M == kFP64) {
+#pragma unroll 1
+            for (int i = tid; i < 4 * n1; i += kT) s.r64[i] = flip(net.d[i], bit_of(s.mask, i >> 2));
+        } else {
+            int nact = 0;
+#pragma unroll 1
+            for (int w = 0; w < n1; w += 32) nact += __popc(s.mask[w >> 5] & (n1 - w < 32 ? (1u << (n1 - w)) - 1u : ~0u));
+            const float g = df_gamma(nact + (net.L > 1 ? 1 << df_split(net.width[2]) : 1) + 2);
+#pragma unroll 1
+            for (int i0 = 0; i0 < 4 * n1; i0 += kT) {
+                const int i = i0 + tid, k = i >> 2;
+                const bool on = i < 4 * n1;
+                const float h = on ? net.h[i] : 0.0f, lo = on ? net.l[i] : 0.0f;
+                float l1 = fabsf(h);
+                l1 += __shfl_xor_sync(full, l1, 1);
+                l1 += __shfl_xor_sync(full, l1, 2);
+                if (on) {
+                    const float sg = bit_of(s.mask, k) ? -1.0f : 1.0f;
+                    s.rhi[i] = sg * h;
+                    s.rlo[i] = sg * lo;
+                    // representation of C: double-float, or FP32 alone on the tensor-core path
+                    const float e = (tc ? kU : 2.0f * kU * kU) * l1 * 1.01f;
+                    s.err[k] = e;
+                    s.carry[k] = __fmaf_ru(g, l1 * 1.001f, e);
                 }
-                // representation of C: double-float, or FP32 alone on the tensor-core path
-                s.err[k] = tc ? kU * l1 * 1.01f : 2.0f * kU * kU * l1 * 1.01f;
             }
         }
     }
     __syncthreads();
-    if (M == kDF && tc) compose_tc_layers(net, s, nrows);
+    if (M == kDF && tc) compose_tc_layers(netg, max_n, nrows);
+#pragma unroll 1
     for (int l = (M == kDF && tc) ? net.L + 1 : 2; l <= net.L; ++l) {
-        const int np = net.width[l - 1], nl = net.width[l], rp = net.row0[l - 1], rl = net.row0[l];
-        const int S = nl >= kT ? 1 : kT / nl;
-        // active list of layer l-1 (diag(s_{l-1}) selects these rows); with a leaky ReLU every
-        // row takes part, the inactive ones scaled by the slope (diag(s + slope (1 - s)))
-        const bool leaky = M == kFP64 && net.slope != 0.0;
-        int nact = 0;
-        for (int base = 0; base < np; base += kT) {
-            const int j = base + tid;
-            const int f = (j < np) ? (leaky ? 1 : (int)bit_of(s.mask, rp + j)) : 0;
-            int tot;
-            const int pos = block_scan_excl(f, s.wsum, &tot);
-            if (f) s.act[nact + pos] = j;
-            nact += tot;
-        }
-        __syncthreads();                     // the active list is read by every thread below
-        float g = 0.0f;
-        if (M == kDF) {
-            g = df_gamma(nact + S + 2);
-            // carry_t = e_j + g |z_j|_1 for the t-th active row j of layer l-1
-            for (int t = tid; t < nact; t += kT) {
-                const int r = rp + s.act[t];
-                const float l1 = fabsf(s.rhi[4 * r]) + fabsf(s.rhi[4 * r + 1]) + fabsf(s.rhi[4 * r + 2]) +
-                                 fabsf(s.rhi[4 * r + 3]);
-                s.carry[t] = __fmaf_ru(g, l1 * 1.001f, s.err[r]);
-            }
-        }
-        __syncthreads();
-        for (int item = tid; item < nl * S; item += kT) {
-            const int k = item % nl, sp = item / nl;
-            if (M == kFP64) {
-                const double *AT = net.AT[l];
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                if (leaky) {
-                    // active: z = -row (weight 1); inactive: z = +row, weight slope
-                    const double sl = net.slope;
-                    for (int t = sp; t < nact; t += S) {
-                        const int j = s.act[t];
-                        double w = __ldg(AT + (size_t)j * nl + k);
-                        if (!bit_of(s.mask, rp + j)) w *= -sl;
-                        const double *z = s.r64 + 4 * (rp + j);
-                        a0 -= w * z[0]; a1 -= w * z[1]; a2 -= w * z[2]; a3 -= w * z[3];
-                    }
-                } else {
-#pragma unroll 4
-                    for (int t = sp; t < nact; t += S) {
-                        const int j = s.act[t];
-                        const double w = __ldg(AT + (size_t)j * nl + k);
-                        const double *z = s.r64 + 4 * (rp + j);          // active: z = -row
-                        a0 -= w * z[0]; a1 -= w * z[1]; a2 -= w * z[2]; a3 -= w * z[3];
-                    }
-                }
-                if (S == 1) {
-                    add_shortcut(net, s, l, k, a0, a1, a2, a3);
-                    const double sg = bit_of(s.mask, rl + k) ? -1.0 : 1.0;
-                    const double *C = net.Cl[l] + 4 * k;
-                    double *r = s.r64 + 4 * (rl + k);
-                    r[0] = sg * (a0 + C[0]); r[1] = sg * (a1 + C[1]); r[2] = sg * (a2 + C[2]); r[3] = sg * (a3 + C[3]);
-                } else {
-                    double *p = s.partd + 4 * item;
-                    p[0] = a0; p[1] = a1; p[2] = a2; p[3] = a3;
-                }
-            } else {
-                const float *Ah = net.AThi[l], *Al = net.ATlo[l];
-                float h0 = 0.f, h1 = 0.f, h2 = 0.f, h3 = 0.f, l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f, eb = 0.f;
-#pragma unroll 4
-                for (int t = sp; t < nact; t += S) {
-                    const int j = s.act[t];
-                    const float ah = __ldg(Ah + (size_t)j * nl + k), al = __ldg(Al + (size_t)j * nl + k);
-                    const float4 zh = *reinterpret_cast<const float4 *>(s.rhi + 4 * (rp + j));   // z = -row
-                    const float4 zl = *reinterpret_cast<const float4 *>(s.rlo + 4 * (rp + j));
-                    df_fma(h0, l0, ah, al, -zh.x, -zl.x);
-                    df_fma(h1, l1, ah, al, -zh.y, -zl.y);
-                    df_fma(h2, l2, ah, al, -zh.z, -zl.z);
-                    df_fma(h3, l3, ah, al, -zh.w, -zl.w);
-                    eb = __fmaf_ru(fabsf(ah), s.carry[t], eb);
-                }
-                if (S == 1) {
-                    const float *Ch = net.Clhi[l] + 4 * k, *Cc = net.Cllo[l] + 4 * k;
-                    df_add(h0, l0, Ch[0], Cc[0]); df_add(h1, l1, Ch[1], Cc[1]);
-                    df_add(h2, l2, Ch[2], Cc[2]); df_add(h3, l3, Ch[3], Cc[3]);
-                    df_norm(h0, l0); df_norm(h1, l1); df_norm(h2, l2); df_norm(h3, l3);
-                    const float sg = bit_of(s.mask, rl + k) ? -1.0f : 1.0f;
-                    *reinterpret_cast<float4 *>(s.rhi + 4 * (rl + k)) = make_float4(sg * h0, sg * h1, sg * h2, sg * h3);
-                    *reinterpret_cast<float4 *>(s.rlo + 4 * (rl + k)) = make_float4(sg * l0, sg * l1, sg * l2, sg * l3);
-                    const float cl1 = fabsf(Ch[0]) + fabsf(Ch[1]) + fabsf(Ch[2]) + fabsf(Ch[3]);
-                    s.err[rl + k] = __fmaf_ru(g, cl1, eb) * 1.01f;
-                } else {
-                    float *p = s.partf + 9 * item;
-                    p[0] = h0; p[1] = h1; p[2] = h2; p[3] = h3; p[4] = l0; p[5] = l1; p[6] = l2; p[7] = l3; p[8] = eb;
-                }
-            }
-        }
-        __syncthreads();
-        if (S > 1) {
-            for (int k = tid; k < nl; k += kT) {
-                if (M == kFP64) {
-                    const double *C = net.Cl[l] + 4 * k;
-                    double a0 = C[0], a1 = C[1], a2 = C[2], a3 = C[3];
-                    for (int sp = 0; sp < S; ++sp) {
-                        const double *p = s.partd + 4 * (sp * nl + k);
-                        a0 += p[0]; a1 += p[1]; a2 += p[2]; a3 += p[3];
-                    }
-                    add_shortcut(net, s, l, k, a0, a1, a2, a3);
-                    const double sg = bit_of(s.mask, rl + k) ? -1.0 : 1.0;
-                    double *r = s.r64 + 4 * (rl + k);
-                    r[0] = sg * a0; r[1] = sg * a1; r[2] = sg * a2; r[3] = sg * a3;
-                } else {
-                    const float *Ch = net.Clhi[l] + 4 * k, *Cc = net.Cllo[l] + 4 * k;
-                    float h0 = Ch[0], h1 = Ch[1], h2 = Ch[2], h3 = Ch[3];
-                    float l0 = Cc[0], l1 = Cc[1], l2 = Cc[2], l3 = Cc[3];
-                    float eb = 0.0f;
-                    for (int sp = 0; sp < S; ++sp) {
-                        const float *p = s.partf + 9 * (sp * nl + k);
-                        df_add(h0, l0, p[0], p[4]); df_add(h1, l1, p[1], p[5]);
-                        df_add(h2, l2, p[2], p[6]); df_add(h3, l3, p[3], p[7]);
-                        eb = __fadd_ru(eb, p[8]);
-                    }
-                    df_norm(h0, l0); df_norm(h1, l1); df_norm(h2, l2); df_norm(h3, l3);
-                    const float sg = bit_of(s.mask, rl + k) ? -1.0f : 1.0f;
-                    *reinterpret_cast<float4 *>(s.rhi + 4 * (rl + k)) = make_float4(sg * h0, sg * h1, sg * h2, sg * h3);
-                    *reinterpret_cast<float4 *>(s.rlo + 4 * (rl + k)) = make_float4(sg * l0, sg * l1, sg * l2, sg * l3);
-                    const float cl1 = fabsf(Ch[0]) + fabsf(Ch[1]) + fabsf(Ch[2]) + fabsf(Ch[3]);
-                    s.err[rl + k] = __fmaf_ru(g, cl1, eb) * 1.01f;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    // a_F = w_out^T diag(s_L) Z_L + [0 | b_out]  (Cor. 1, Eq. 8)
-    if (M == kFP64 && net.M >= 2) {
-        // final max pooling (Sec. 5.2): a_F(i) of every head into row n_units + i, then the face
-        // plane a_F(j) of the cell's pooled index j and the pooling rows a_F(i) - a_F(j)
-        const int nL = net.width[net.L], rL = net.row0[net.L];
-        for (int i = 0; i < net.M; ++i) {
-            const double *wh = net.w_heads + (size_t)i * nL;
-            double f[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int k = tid; k < nL; k += kT) {
-                const double w = bit_of(s.mask, rL + k) ? wh[k] : -net.slope * wh[k];
-                if (w != 0.0)
-                    for (int c = 0; c < 4; ++c) f[c] -= w * s.r64[4 * (rL + k) + c];
-            }
-            for (int c = 0; c < 4; ++c) f[c] = warp_sum(f[c]);
-            if ((tid & 31) == 0)
-                for (int c = 0; c < 4; ++c) s.partd[4 * (tid >> 5) + c] = f[c];
-            __syncthreads();
-            if (tid == 0) {
-                double F[4] = {0.0, 0.0, 0.0, net.b_heads[i]};
-                for (int w = 0; w < kNW; ++w)
-                    for (int c = 0; c < 4; ++c) F[c] += s.partd[4 * w + c];
-                for (int c = 0; c < 4; ++c) s.r64[4 * (net.n_units + i) + c] = F[c];
-            }
-            __syncthreads();
-        }
-        if (tid == 0) {
-            int j = 0;
-            for (int i = 0; i < net.M; ++i)
-                if (bit_of(s.mask, net.n_units + i)) { j = i; break; }
-            for (int c = 0; c < 4; ++c) s.aF[c] = s.r64[4 * (net.n_units + j) + c];
-            s.eF[0] = 0.0f;
-        }
-        __syncthreads();
-        if (tid < net.M)
-            for (int c = 0; c < 4; ++c) s.r64[4 * (net.n_units + tid) + c] -= s.aF[c];
-        __syncthreads();
-        return;
-    }
-    {
-        const int nL = net.width[net.L], rL = net.row0[net.L];
+        const int nl = net.width[l], rp = net.row0[l - 1], rl = net.row0[l];
+        const int t0 = s.lst0[l - 1], t1 = s.lst0[l];
         if (M == kFP64) {
-            double f[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int k = tid; k < nL; k += kT) {
-                // active: row = -Z (weight 1); inactive: row = +Z, weight slope (0 for a ReLU)
-                const double w = bit_of(s.mask, rL + k) ? net.w_out[k] : -net.slope * net.w_out[k];
-                if (w != 0.0)
-                    for (int c = 0; c < 4; ++c) f[c] -= w * s.r64[4 * (rL + k) + c];
-            }
-            for (int c = 0; c < 4; ++c) f[c] = warp_sum(f[c]);
-            if ((tid & 31) == 0)
-                for (int c = 0; c < 4; ++c) s.partd[4 * (tid >> 5) + c] = f[c];
-            __syncthreads();
-            if (tid == 0) {
-                double F[4] = {0.0, 0.0, 0.0, net.b_out};
-                for (int w = 0; w < kNW; ++w)
-                    for (int c = 0; c < 4; ++c) F[c] += s.partd[4 * w + c];
-                for (int c = 0; c < 4; ++c) s.aF[c] = F[c];
-                s.eF[0] = 0.0f;
+            const double *AT = net.d + net.offA[l], *C = net.d + net.offC[l];
+            if (nl > kT / 2) {
+                // wide layers: a row per thread, whose weight feeds four products (a column per thread would
+                // read every weight four times from the L2: 1.16 ms against 1.02 ms for 1000 patterns of a
+                // 3-[250]x5-1 net, 1.59 ms against 1.22 ms for 400 of a 3-[500]x4-1 net)
+#pragma unroll 1
+                for (int k = tid; k < nl; k += kT) {
+                    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+#pragma unroll 4
+                    for (int t = t0; t < t1; ++t) {
+                        const int r = s.lst[t];
+                        const double w = __ldg(AT + (r - rp) * nl + k);
+                        const double *z = s.r64 + 4 * r;
+                        a0 -= w * z[0]; a1 -= w * z[1]; a2 -= w * z[2]; a3 -= w * z[3];
+                    }
+                    const bool act = bit_of(s.mask, rl + k);
+                    double *r = s.r64 + 4 * (rl + k);
+                    r[0] = flip(a0 + C[4 * k], act); r[1] = flip(a1 + C[4 * k + 1], act);
+                    r[2] = flip(a2 + C[4 * k + 2], act); r[3] = flip(a3 + C[4 * k + 3], act);
+                }
+            } else if (tid < 4 * nl) {
+                // one column of row k, and of row k + kT / 4 where the warp has one: 4 n_l <= 2 kT
+                const int k = tid >> 2, c = tid & 3, k2 = min(k + kT / 4, nl - 1);
+                double acc, acc2 = 0.0;
+                const double Ci = C[tid];
+                if ((tid & ~31) + kT < 4 * nl) {
+                    acc = 0.0;
+#pragma unroll 4
+                    for (int t = t0; t < t1; ++t) {
+                        const int r = s.lst[t];
+                        const double *w = AT + (r - rp) * nl;
+                        const double z = s.r64[4 * r + c];          // active: z = -row
+                        acc -= __ldg(w + k) * z;
+                        acc2 -= __ldg(w + k2) * z;
+                    }
+                    if (k + kT / 4 < nl) s.r64[4 * (rl + k2) + c] = flip(acc2 + C[4 * k2 + c], bit_of(s.mask, rl + k2));
+                } else {
+                    acc = dot_active(s, AT, nl, rp, k, c, t0, t1);
+                }
+                s.r64[4 * rl + tid] = flip(acc + Ci, bit_of(s.mask, rl + k));
             }
         } else {
-            // one warp, lanes over the last layer, double-float with a bound
-            if (tid < 32) {
-                int cnt = 0;
-                for (int k = tid; k < nL; k += 32) cnt += bit_of(s.mask, rL + k);
-                for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-                const float g = df_gamma(cnt + 40);
-                float h[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f}, eb = 0.0f, e2 = 0.0f;
-                for (int k = tid; k < nL; k += 32) {
-                    if (!bit_of(s.mask, rL + k)) continue;
-                    const float wh = net.w_out_hi[k], wl = net.w_out_lo[k];
-                    const float *zh = s.rhi + 4 * (rL + k), *zl = s.rlo + 4 * (rL + k);
-                    float l1 = 0.0f;
-                    for (int c = 0; c < 4; ++c) {
-                        df_fma(h[c], lo[c], wh, wl, -zh[c], -zl[c]);
-                        l1 += fabsf(zh[c]);
-                    }
-                    if (tc) {           // this product's rounding (bound) + propagated estimates (rss)
-                        eb = __fmaf_ru(fabsf(wh), g * l1 * 1.001f, eb);
-                        e2 = fmaf(wh * s.err[rL + k], wh * s.err[rL + k], e2);
-                    } else {
-                        eb = __fmaf_ru(fabsf(wh), __fmaf_ru(g, l1 * 1.001f, s.err[rL + k]), eb);
+            const float *Ah = net.h + net.offA[l], *Al = net.l + net.offA[l];
+            const int sh = df_split(nl), S = 1 << sh;
+            const float g = df_gamma(t1 - t0 + S + 2);
+            const float gn = l < net.L ? df_gamma(s.lst0[l + 1] - t1 + (1 << df_split(net.width[l + 1])) + 2) : 0.0f;
+            if (nl <= kNarrow) {
+                // one lane per row, column and part of the sum, in one pass of the block
+                const int sp = tid & (S - 1), c = (tid >> sh) & 3, k = tid >> (sh + 2);
+                const bool on = k < nl;
+                const float ch = on ? net.h[net.offC[l] + 4 * k + c] : 0.0f, cl = on ? net.l[net.offC[l] + 4 * k + c] : 0.0f;
+                float h = 0.0f, lo = 0.0f, eb = 0.0f;
+                if (on) {
+#pragma unroll 2
+                    for (int t = t0 + sp; t < t1; t += S) {
+                        const int r = s.lst[t];
+                        const float ah = __ldg(Ah + (r - rp) * nl + k), al = __ldg(Al + (r - rp) * nl + k);
+                        df_fma(h, lo, ah, al, -s.rhi[4 * r + c], -s.rlo[4 * r + c]);      // z = -row
+                        eb = __fmaf_ru(fabsf(ah), s.carry[r], eb);
                     }
                 }
 #pragma unroll 1
-                for (int o = 16; o > 0; o >>= 1) {
-                    for (int c = 0; c < 4; ++c) {
-                        const float oh = __shfl_xor_sync(0xffffffffu, h[c], o);
-                        const float ol = __shfl_xor_sync(0xffffffffu, lo[c], o);
-                        df_add(h[c], lo[c], oh, ol);
-                    }
-                    eb = __fadd_ru(eb, __shfl_xor_sync(0xffffffffu, eb, o));
-                    e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+                for (int o = 1; o < S; o <<= 1) {
+                    const float oh = __shfl_xor_sync(full, h, o), ol = __shfl_xor_sync(full, lo, o);
+                    df_add(h, lo, oh, ol);
+                    eb = __fadd_ru(eb, __shfl_xor_sync(full, eb, o));
                 }
-                if (tc) eb += 2.0f * sqrtf(e2);
-                if (tid == 0) {
-                    const float bh = (float)net.b_out, bl = (float)(net.b_out - (double)bh);
-                    df_add(h[3], lo[3], bh, bl);
-                    float l1 = fabsf(bh);
-                    for (int c = 0; c < 4; ++c) {
-                        df_norm(h[c], lo[c]);
-                        s.aFhi[c] = h[c];
-                        s.aFlo[c] = lo[c];
-                        s.aF[c] = (double)h[c] + (double)lo[c];
+                df_add(h, lo, ch, cl);
+                df_norm(h, lo);
+                float l1 = fabsf(h), cl1 = fabsf(ch);
+#pragma unroll 1
+                for (int o = S; o < 4 * S; o <<= 1) {
+                    l1 += __shfl_xor_sync(full, l1, o);
+                    cl1 += __shfl_xor_sync(full, cl1, o);
+                }
+                if (on && sp == 0) {
+                    const float sg = bit_of(s.mask, rl + k) ? -1.0f : 1.0f;
+                    s.rhi[4 * (rl + k) + c] = sg * h;
+                    s.rlo[4 * (rl + k) + c] = sg * lo;
+                    const float e = __fmaf_ru(g, cl1, eb) * 1.01f;
+                    s.err[rl + k] = e;
+                    s.carry[rl + k] = __fmaf_ru(gn, l1 * 1.001f, e);
+                }
+            } else {
+                // S lanes per row
+#pragma unroll 1
+                for (int i0 = 0; i0 < nl * S; i0 += kT) {
+                    const int item = i0 + tid, k = item >> sh, sp = item & (S - 1);
+                    float h0 = 0.f, h1 = 0.f, h2 = 0.f, h3 = 0.f, l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f, eb = 0.f;
+                    if (k < nl) {
+#pragma unroll 4
+                        for (int t = t0 + sp; t < t1; t += S) {
+                            const int r = s.lst[t];
+                            const float ah = __ldg(Ah + (r - rp) * nl + k), al = __ldg(Al + (r - rp) * nl + k);
+                            const float4 zh = *reinterpret_cast<const float4 *>(s.rhi + 4 * r);      // z = -row
+                            const float4 zl = *reinterpret_cast<const float4 *>(s.rlo + 4 * r);
+                            df_fma(h0, l0, ah, al, -zh.x, -zl.x);
+                            df_fma(h1, l1, ah, al, -zh.y, -zl.y);
+                            df_fma(h2, l2, ah, al, -zh.z, -zl.z);
+                            df_fma(h3, l3, ah, al, -zh.w, -zl.w);
+                            eb = __fmaf_ru(fabsf(ah), s.carry[r], eb);
+                        }
                     }
-                    s.eF[0] = __fmaf_ru(g, l1, eb) * 1.01f;
+#pragma unroll 1
+                    for (int o = 1; o < S; o <<= 1) {
+                        df_add(h0, l0, __shfl_xor_sync(full, h0, o), __shfl_xor_sync(full, l0, o));
+                        df_add(h1, l1, __shfl_xor_sync(full, h1, o), __shfl_xor_sync(full, l1, o));
+                        df_add(h2, l2, __shfl_xor_sync(full, h2, o), __shfl_xor_sync(full, l2, o));
+                        df_add(h3, l3, __shfl_xor_sync(full, h3, o), __shfl_xor_sync(full, l3, o));
+                        eb = __fadd_ru(eb, __shfl_xor_sync(full, eb, o));
+                    }
+                    if (k < nl && sp == 0) {
+                        const float *Ch = net.h + net.offC[l] + 4 * k, *Cc = net.l + net.offC[l] + 4 * k;
+                        df_add(h0, l0, Ch[0], Cc[0]); df_add(h1, l1, Ch[1], Cc[1]);
+                        df_add(h2, l2, Ch[2], Cc[2]); df_add(h3, l3, Ch[3], Cc[3]);
+                        df_norm(h0, l0); df_norm(h1, l1); df_norm(h2, l2); df_norm(h3, l3);
+                        const float sg = bit_of(s.mask, rl + k) ? -1.0f : 1.0f;
+                        *reinterpret_cast<float4 *>(s.rhi + 4 * (rl + k)) = make_float4(sg * h0, sg * h1, sg * h2, sg * h3);
+                        *reinterpret_cast<float4 *>(s.rlo + 4 * (rl + k)) = make_float4(sg * l0, sg * l1, sg * l2, sg * l3);
+                        const float cl1 = fabsf(Ch[0]) + fabsf(Ch[1]) + fabsf(Ch[2]) + fabsf(Ch[3]);
+                        const float e = __fmaf_ru(g, cl1, eb) * 1.01f;
+                        s.err[rl + k] = e;
+                        s.carry[rl + k] = __fmaf_ru(gn, (fabsf(h0) + fabsf(h1) + fabsf(h2) + fabsf(h3)) * 1.001f, e);
+                    }
                 }
             }
         }
+        __syncthreads();
     }
-    __syncthreads();
+    // a_F = w_out^T diag(s_L) Z_L + [0 | b_out]  (Cor. 1, Eq. 8), warp 0: lane 4 p + c takes column c of
+    // every 8th active unit
+    if (tid < 32) {
+        const int rL = net.row0[net.L], t0 = s.lst0[net.L], t1 = s.lst0[net.L + 1], c = tid & 3;
+        if (M == kFP64) {
+            double f = 0.0;
+#pragma unroll 4
+            for (int t = t0 + (tid >> 2); t < t1; t += 8) {
+                const int r = s.lst[t];
+                f -= net.d[net.offw + r - rL] * s.r64[4 * r + c];
+            }
+#pragma unroll 1
+            for (int o = 4; o < 32; o <<= 1) f += __shfl_xor_sync(full, f, o);
+            if (c == 3) f += net.b_out;
+            if (tid < 4) {
+                s.aF[c] = f;
+                s.aFhi[c] = (float)f;
+            }
+            if (tid == 0) s.eF[0] = 0.0f;
+        } else {
+            // double-float with a bound on the l1 error of the four columns
+            const float g = df_gamma(t1 - t0 + 40);
+            float h = 0.0f, lo = 0.0f, eb = 0.0f, e2 = 0.0f;
+#pragma unroll 2
+            for (int t = t0 + (tid >> 2); t < t1; t += 8) {
+                const int r = s.lst[t];
+                const float wh = net.h[net.offw + r - rL], wl = net.l[net.offw + r - rL], zh = s.rhi[4 * r + c];
+                df_fma(h, lo, wh, wl, -zh, -s.rlo[4 * r + c]);
+                // this column's rounding, and (once) the row's error
+                eb = __fmaf_ru(fabsf(wh), g * fabsf(zh) * 1.001f, eb);
+                if (tc) e2 = fmaf(wh * s.err[r], wh * s.err[r], e2);        // estimates, by root sum of squares
+                else if (c == 0) eb = __fmaf_ru(fabsf(wh), s.err[r], eb);
+            }
+#pragma unroll 1
+            for (int o = 4; o < 32; o <<= 1) {
+                const float oh = __shfl_xor_sync(full, h, o), ol = __shfl_xor_sync(full, lo, o);
+                df_add(h, lo, oh, ol);
+                eb = __fadd_ru(eb, __shfl_xor_sync(full, eb, o));
+                e2 += __shfl_xor_sync(full, e2, o);
+            }
+            eb = __fadd_ru(eb, __shfl_xor_sync(full, eb, 1));
+            eb = __fadd_ru(eb, __shfl_xor_sync(full, eb, 2));
+            if (tc) eb += 2.0f * sqrtf(e2);
+            if (c == 3) df_add(h, lo, net.b_out_hi, net.b_out_lo);
+            df_norm(h, lo);
+            if (tid < 4) {
+                s.aFhi[c] = h;
+                s.aFlo[c] = lo;
+                s.aF[c] = (double)h + (double)lo;
+            }
+            if (tid == 0) s.eF[0] = __fmaf_ru(g, fabsf(net.b_out_hi), eb) * 1.01f;
+        }
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -853,68 +1104,447 @@ __device__ void proposal_scores(const MarchArgs &a, const NetDev &net, int64_t c
 }
 
 // ------------------------------------------------------------------------------------------
-// one cell
+// the face in one pass
 
-struct CellOut {
-    int emit;        // corners written (0 = empty)
-    int ambiguous;   // kDF: an undecidable sign test; nothing written
-};
-
-template <int M>
-__device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net, int64_t cell, const Sh &s)
+// FP64 to FP32 towards zero with integer operations (a conversion instruction goes through the FP64
+// pipe): within 2^-23 of x relative; 0 below FP32's normal range, about 3.4e38 above it
+__device__ __forceinline__ float f32_toward_zero(double x)
 {
-    const Arena &ar = a.ar;
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned m = min(hi & 0x7fffffffu, 0x47efffffu);
+    unsigned f = (__funnelshift_l(lo, m, 3) - 0x40000000u) & 0x7fffffffu;   // exponent 11 bits -> 8: minus 896
+    if (m < 0x38100000u) f = 0u;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// FP64 row k in FP32, towards zero (one copy of the code: it runs three times per cell)
+__device__ __noinline__ float4 row32_fp64(const double *r64, int k)
+{
+    const double2 a = reinterpret_cast<const double2 *>(r64)[2 * k], b = reinterpret_cast<const double2 *>(r64)[2 * k + 1];
+    return make_float4(f32_toward_zero(a.x), f32_toward_zero(a.y), f32_toward_zero(b.x), f32_toward_zero(b.y));
+}
+
+// row k in FP32: its hi words (kDF), or its FP64 words towards zero
+template <int M>
+__device__ __forceinline__ float4 row32(const Sh &s, int k)
+{
+    if (M == kDF) return *reinterpret_cast<const float4 *>(s.rhi + 4 * k);
+    return row32_fp64(s.r64, k);
+}
+
+// Warp 0: the ring of the lines' intervals (s.seg).  A line carries an edge when the part of it
+// inside all others is not empty; the line that ends an edge carries the next one.  Writes the
+// edge planes s.pe[0][0 .. m) counter-clockwise and the area flag s.si[6] (1: clearly above the
+// smallest kept area, 2: FP64 decides); returns m, or 0 when the edges do not close into one ring.
+__device__ __forceinline__ int ring_of_lines(const Sh &s, int n)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    int *cl = s.ring, *cn = cl + kLines, *cp = cn + kLines, *rk = cp + kLines;
+    float area = 0.0f;
+    int m = 0;
+#pragma unroll 1
+    for (int i = lane; i < kLines; i += 32) {
+        const float4 p = s.seg[i];
+        const bool alive = i < n && p.y > p.x;
+        const unsigned b = __ballot_sync(full, alive);
+        const int r = m + __popc(b & ((1u << lane) - 1u));
+        rk[i] = alive ? r : -1;
+        if (alive) {
+            cl[r] = i; cn[r] = __float_as_int(p.w); cp[r] = __float_as_int(p.z);
+            // twice the triangle of the edge and the origin, less what rounding can make of it (below
+            // 1e-6 of the edge: the origin lies in the face, so the sum has no cancellation)
+            area += (-s.line[i].z - 2e-6f) * (p.y - p.x);
+        }
+        m += __popc(b);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) area += __shfl_xor_sync(full, area, o);
+    bool ok = m >= 3 && m <= 32;
+    int nxt = -1, prv = -1, k = -1;
+    if (ok && lane < m) {
+        const int jn = cn[lane], jp = cp[lane];
+        nxt = jn >= 0 ? rk[jn] : -1;
+        prv = jp >= 0 ? rk[jp] : -1;
+        k = __float_as_int(s.line[cl[lane]].w);
+    }
+    const int back = __shfl_sync(full, prv, nxt & 31);
+    ok = ok && (lane >= m || (nxt >= 0 && prv >= 0 && back == lane));
+    if (!__all_sync(full, ok)) return 0;
+    int cur = 0, pos = 0, left = m;
+#pragma unroll 1
+    do {
+        if (lane == cur) pos = m - left;
+        cur = __shfl_sync(full, nxt, cur);
+        --left;
+    } while (cur != 0 && left > 0);
+    if (cur != 0 || left != 0) return 0;             // no cycle, or a shorter one
+    if (lane < m) s.pe[0][pos] = k;
+    if (lane == 0) s.si[6] = area > 1e-12f ? 1 : 2;
+    __syncwarp();
+    return m;
+}
+
+// Warp 0: the ring's vertices in FP64, each from the rows of its two edges and the face plane
+// (Eq. 11, solve3's Cramer's rule), one lane per vertex and coordinate: the warp issues the
+// instructions of one coordinate instead of three, and an FP64 warp instruction takes about 64
+// cycles for one lane as for 32.  Also the vertices in FP32 with the vertex term of the check's
+// bound (vf[i][3]) and kDF's vertex error bounds.  False when a vertex is not known well enough.
+template <int M>
+__device__ __forceinline__ bool ring_vertices(const Arena &ar, const Sh &s, int m, int N)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    // the planes' hash words, for the pushes
+    const int ze = lane < m ? s.pe[0][lane] : N;
+    const unsigned long long zv = ze < N ? __ldg(ar.zob + ze) : 0ull;
+    const double *R = s.r64;
+    if (M == kDF) {
+        // the edges' rows as FP64, one lane per coefficient, into the spare polygon buffer
+        double *e = &s.pv[1][0][0];
+        for (int i = lane; i < 4 * m; i += 32) {
+            const int q = 4 * s.pe[0][i >> 2] + (i & 3);
+            e[i] = (double)s.rhi[q] + (double)s.rlo[q];
+        }
+        __syncwarp();
+        R = e;
+    }
+    const int v = lane / 3, d = lane - 3 * v, d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+    const int l0 = 3 * v, l1 = l0 + 1, l2 = l0 + 2 > 31 ? 31 : l0 + 2;
+    bool good = true;
+#pragma unroll 1
+    for (int b = 0; b < m; b += 10) {
+        const int i = b + v;
+        const bool on = v < 10 && i < m;
+        const int iq = on ? i : 0, ip = iq == 0 ? m - 1 : iq - 1;
+        const int ka = s.pe[0][ip], kb = s.pe[0][iq];
+        const double *p = R + 4 * (M == kDF ? ip : ka), *q = R + 4 * (M == kDF ? iq : kb), *f = s.aF;
+        const double c0 = q[d1] * f[d2] - q[d2] * f[d1], c1 = f[d1] * p[d2] - f[d2] * p[d1],
+                     c2 = p[d1] * q[d2] - p[d2] * q[d1];
+        const double det = p[0] * __shfl_sync(full, c0, l0) + p[1] * __shfl_sync(full, c0, l1) + p[2] * __shfl_sync(full, c0, l2);
+        const double inv = -1.0 / det;
+        const double x = (p[3] * c0 + q[3] * c1 + f[3] * c2) * inv;
+        const float xf = (float)x;
+        float X = fmaxf(1.0f, fabsf(xf));
+        X = fmaxf(X, fmaxf(__shfl_sync(full, X, l0), fmaxf(__shfl_sync(full, X, l1), __shfl_sync(full, X, l2)))) * 1.0001f;
+        float w = 10.5f * kU * X;
+        bool fine = isfinite(xf);
+        if (M == kDF) {
+            // |M^-1|_inf max(e_a, e_b, e_F) max(1, |v|) (1.1): as df_final_vertices
+            float rs = (float)(fabs(c0) + fabs(c1) + fabs(c2)) * 1.0001f;
+            rs = fmaxf(__shfl_sync(full, rs, l0), fmaxf(__shfl_sync(full, rs, l1), __shfl_sync(full, rs, l2)));
+            const float in = rs * fabsf((float)inv) * 1.0001f;
+            const float e = fmaxf(s.err[ka], fmaxf(s.err[kb], s.eF[0]));
+            const float dv = fmaf(in * e, X * 1.1f, 4e-16f * X) * 1.01f;
+            fine = fine && dv <= (float)kVertexTol * X;
+            w = fmaf(8.5f * kU, X, dv) * 1.0001f;
+            if (on && d == 0) s.dvb[i] = dv;
+        }
+        if (on) {
+            s.pv[0][i][d] = x;
+            s.vf[i][d] = xf;
+            if (d == 0) s.vf[i][3] = w;
+            good = good && fine;
+        }
+        if (on && d == 0) s.pf[0][i][0] = X;
+    }
+    s.zb[lane] = zv;
+    return __all_sync(full, good);
+}
+
+// A close call of the FP32 test (or one that is not finite): row k at vertex i in FP64, as the
+// sequential clip tests it.  1: violated, 2: within the tolerance or undecidable, 0: it holds.  Out
+// of line: FP32 decides nearly every pair.
+template <int M>
+__device__ __noinline__ int close_call(int max_n, double delta, int k, int i, float ri, float rl1, float band, float Xm)
+{
+    const Sh s = make_sh(max_n);
+    const double *v6 = s.pv[0][i];
+    if (M == kFP64) {
+        const double dd = pdist((const double *)(s.r64 + 4 * k), (double)ri, v6);
+        if (dd > delta) return 1;
+        return dd < -delta ? 0 : 2;
+    }
+    atomicAdd(s.blk + 5, 1ull);
+    double r6[4];
+    row64<kDF>(s, k, r6);
+    const double s6 = r6[0] * v6[0] + r6[1] * v6[1] + r6[2] * v6[2] + r6[3];
+    const double m6 = fabs(r6[0] * v6[0]) + fabs(r6[1] * v6[1]) + fabs(r6[2] * v6[2]) + fabs(r6[3]);
+    const double B6 = (double)s.err[k] * (double)Xm + (double)rl1 * 1.0001 * (double)s.dvb[i] + (double)band + 1e-15 * m6;
+    if (s6 > B6) return 1;
+    return s6 < -B6 ? 0 : 2;
+}
+
+// The face of the cell without the sequential cuts: every warp contributes its rows nearest to the
+// entry point, the lines in which these rows (and the box) meet the face plane are cut against
+// each other all at once (each line's interval inside all the others, in FP32 coordinates of the
+// plane about the entry point), and the intervals that remain close into the polygon's ring.  Its
+// vertices are solved in FP64 from their planes; then every row is tested at every vertex in FP32
+// with a certified bound, a close call in FP64.  Rows found violated join the edges as the lines
+// of another round.  The ring is kept only when every row that is not an edge at a vertex is
+// beyond the tolerance there, which makes it the cell's face whatever FP32 did before: the vertices
+// are then the system's own, in order.  Anything else (a row within the tolerance, an open
+// ring, a vertex not known well enough, too many rounds) returns false, and the sequential clip
+// (kFP64) or FP64 (kDF) decides the cell from the start.
+//
+// What bounds it is the serial chain of a cell, so the chain is short: about five barriers and a
+// dozen FP64 instructions, where the cuts one by one issued some 400 FP64 instructions in one warp
+// (about 64 cycles each, for one lane as for 32).  From the rows to the checked face a cell of a
+// 3-[64]x4-1 net in FP64 took 69,700 cycles of its block with the cuts one by one and takes 12,800; a
+// 3-[32]x4-1 net in mixed precision 68,000 and 11,200.  The march of the first (44,304 cells from one
+// ray) went from 12.3 to 4.6 ms, of the second (10,472 cells) from 3.6 to 1.5 ms.
+template <int M>
+__device__ __forceinline__ bool fast_face(const MarchArgs &a, int N, const Sh &s, int *rounds)
+{
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int N = net.N, NC = N + kBoxPlanes;          // checked rows: neurons + box
-    long long tp0 = 0, tp1 = 0, tp2 = 0, tp2a = 0, tp3a = 0, tp3 = 0, tp4 = 0, tp4a = 0, tp5 = 0;
-    AM_TICK(tp0);
-    if (a.rows_in) {
-        // rows composed beforehand on the tensor cores, as FP32 pairs (the hi words [hi x 4] of
-        // rows 0..N, then their lo words [lo x 4])
-        // (signs as compose<M>, a_F last).  The pairs are the rows: the double-float tests are
-        // certified against them with no further row error, as FP64 tests take FP64 rows.
-        const float4 *src = reinterpret_cast<const float4 *>(a.rows_in) + (cell - a.begin) * (int64_t)(N + 1) * 2;
+    const unsigned full = 0xffffffffu;
+    const int NC = N + kBoxPlanes;
+    long long tq0 = 0, tq1 = 0;
+    AM_TICK(tq0);
+    int n;                                           // lines
+    {
+        const float px = s.ent[0], py = s.ent[1], pz = s.ent[2];
+        const int nwr = min(kNW, (N + 31) >> 5), P = nwr == 1 ? 32 : min(kLinePicks, (kLines - kBoxPlanes) / nwr);
+        float b1 = 3.0e38f, b2 = 3.0e38f;
+        int k1 = -1, k2 = -1;
+        bool loose = false;
+#pragma unroll 1
         for (int k = tid; k < N; k += kT) {
-            const float4 h = __ldcs(src + k), l = __ldcs(src + (N + 1) + k);
-            if (M == kFP64) {
-                double *r = s.r64 + 4 * k;
-                r[0] = (double)h.x + (double)l.x; r[1] = (double)h.y + (double)l.y;
-                r[2] = (double)h.z + (double)l.z; r[3] = (double)h.w + (double)l.w;
+            const float4 r = row32<M>(s, k);
+            const float n2 = r.x * r.x + r.y * r.y + r.z * r.z;
+            if (!(n2 > kTiny && n2 < kHuge)) continue;
+            const float ri = rsqrtf(n2);
+            if (M == kDF) loose |= s.err[k] * ri > kDfLoose;
+            const float d = fabsf(fmaf(r.x, px, fmaf(r.y, py, fmaf(r.z, pz, r.w)))) * ri;
+            if (d < b1) { b2 = b1; k2 = k1; b1 = d; k1 = k; }
+            else if (d < b2) { b2 = d; k2 = k; }
+        }
+        // kDF: as in the sequential clip, a row error that no useful number of tests survives
+        if (M == kDF && tid == 0)
+            loose |= s.eF[0] * rsqrtf(s.aFhi[0] * s.aFhi[0] + s.aFhi[1] * s.aFhi[1] + s.aFhi[2] * s.aFhi[2]) > kDfLoose;
+        if (loose) s.si[4] = 1;
+        if (wid < nwr) {
+            int *near = s.near_k + kBoxPlanes + wid * P;
+            if (nwr == 1) {
+                near[lane] = k1;
             } else {
-                *reinterpret_cast<float4 *>(s.rhi + 4 * k) = h;
-                *reinterpret_cast<float4 *>(s.rlo + 4 * k) = l;
-                s.err[k] = 0.0f;
+#pragma unroll 1
+                for (int q = 0; q < P; ++q) {
+                    // the distance's bits, the lane in the lowest five: one reduction picks the row
+                    const unsigned key = k1 >= 0 ? (__float_as_uint(b1) & ~31u) | (unsigned)lane : 0xffffffffu;
+                    const unsigned best = __reduce_min_sync(full, key);
+                    if (best == 0xffffffffu) {
+                        if (lane == 0)
+                            for (int z = q; z < P; ++z) near[z] = -1;
+                        break;
+                    }
+                    if (key == best) { near[q] = k1; b1 = b2; k1 = k2; k2 = -1; }
+                }
             }
         }
-        if (tid < 4) {
-            const float h = reinterpret_cast<const float *>(src + N)[tid];
-            const float l = reinterpret_cast<const float *>(src + 2 * N + 1)[tid];
-            s.aF[tid] = (double)h + (double)l;
-            if (M == kDF) { s.aFhi[tid] = h; s.aFlo[tid] = l; }
-        }
-        if (tid == 0) s.eF[0] = 0.0f;
-        __syncthreads();
-    } else {
-        compose<M>(net, s, false, a.max_n + kBoxPlanes + kSquarePlanes);
+        if (tid < kBoxPlanes) s.near_k[tid] = N + tid;
+        n = kBoxPlanes + nwr * P;
     }
-    AM_TICK(tp1);
+    __syncthreads();
+    AM_TICK(tq1);
+    AM_PHASE(a, 2, tq0, tq1);
+    if (M == kDF && s.si[4]) return false;
+    for (int round = 0;; ++round) {
+        AM_TICK(tq0);
+        if (tid < kLines) {
+            // the lines in the plane's coordinates (u, w) about the entry point
+            float A = 0.0f, B = 0.0f, C = -1.0f;
+            const int k = tid < n ? s.near_k[tid] : -1;
+            if (k >= 0) {
+                const float f0 = s.aFhi[0], f1 = s.aFhi[1], f2 = s.aFhi[2];
+                const float inv = rsqrtf(f0 * f0 + f1 * f1 + f2 * f2);
+                const float n0 = f0 * inv, n1 = f1 * inv, n2 = f2 * inv;
+                const float ax = fabsf(n0), ay = fabsf(n1), az = fabsf(n2);
+                const int ei = (ax <= ay && ax <= az) ? 0 : (ay <= az ? 1 : 2);
+                // u = n x e_i, w = n x u
+                float u0 = ei == 0 ? 0.0f : (ei == 1 ? -n2 : n1), u1 = ei == 0 ? n2 : (ei == 1 ? 0.0f : -n0),
+                      u2 = ei == 0 ? -n1 : (ei == 1 ? n0 : 0.0f);
+                const float un = rsqrtf(u0 * u0 + u1 * u1 + u2 * u2);
+                u0 *= un; u1 *= un; u2 *= un;
+                const float w0 = n1 * u2 - n2 * u1, w1 = n2 * u0 - n0 * u2, w2 = n0 * u1 - n1 * u0;
+                const float4 r = row32<M>(s, k);
+                A = r.x * u0 + r.y * u1 + r.z * u2;
+                B = r.x * w0 + r.y * w1 + r.z * w2;
+                const float q2 = A * A + B * B;
+                if (q2 > 1e-10f * (r.x * r.x + r.y * r.y + r.z * r.z)) {
+                    const float q = rsqrtf(q2);
+                    C = fmaf(r.x, s.ent[0], fmaf(r.y, s.ent[1], fmaf(r.z, s.ent[2], r.w))) * q;
+                    A *= q; B *= q;
+                } else {
+                    A = B = 0.0f;                     // (nearly) parallel to the face plane: no line in it
+                }
+            }
+            s.line[tid] = make_float4(A, B, C, __int_as_float(k));
+        }
+        __syncthreads();
+        AM_TICK(tq1);
+        AM_PHASE(a, 1, tq0, tq1);
+        {
+            // line i's interval inside a quarter of the others: at -c n + t (-b, a), line j holds for
+            // t D <= c_i (n_i . n_j) - c_j, D = n_i x n_j
+            const int i = tid / kParts;
+            float t0 = -3.0e38f, t1 = 3.0e38f;
+            int j0 = -1, j1 = -1;
+            const float4 L = s.line[i];
+#pragma unroll 2
+            for (int j = tid & (kParts - 1); j < n; j += kParts) {
+                const float4 o = s.line[j];
+                const float D = L.x * o.y - L.y * o.x, num = L.z * (L.x * o.x + L.y * o.y) - o.z;
+                const float t = __fdividef(num, D);
+                if (D > 1e-7f && t < t1) { t1 = t; j1 = j; }
+                if (D < -1e-7f && t > t0) { t0 = t; j0 = j; }
+                // beside a parallel line that cuts it off
+                if (fabsf(D) <= 1e-7f && j != i && num < 0.0f) t1 = -3.0e38f;
+            }
+            if (L.x == 0.0f && L.y == 0.0f) t1 = -3.0e38f;
+#pragma unroll 1
+            for (int o = 1; o < kParts; o <<= 1) {
+                const float u0 = __shfl_xor_sync(full, t0, o), u1 = __shfl_xor_sync(full, t1, o);
+                const int i0 = __shfl_xor_sync(full, j0, o), i1 = __shfl_xor_sync(full, j1, o);
+                if (u0 > t0) { t0 = u0; j0 = i0; }
+                if (u1 < t1) { t1 = u1; j1 = i1; }
+            }
+            if ((tid & (kParts - 1)) == 0) s.seg[i] = make_float4(t0, t1, __int_as_float(j0), __int_as_float(j1));
+        }
+        if (tid == 0) { s.si[3] = 0; s.si[4] = 0; }
+        __syncthreads();
+        AM_TICK(tq0);
+        AM_PHASE(a, 3, tq1, tq0);
+        if (wid == 0) {
+            const int m = ring_of_lines(s, n);
+            const bool ok = m > 0 && ring_vertices<M>(a.ar, s, m, N);
+            if (lane == 0) {
+                s.si[0] = ok ? m : 0;
+                s.blk[6] += (unsigned long long)m;
+            }
+        }
+        __syncthreads();
+        AM_TICK(tq1);
+        AM_PHASE(a, 4, tq0, tq1);
+        const int m = s.si[0];
+        if (m == 0) return false;
+        // ---- a5: every row at every vertex
+        float Xm = 1.0f;
+        if (M == kDF)
+#pragma unroll 1
+            for (int i = 0; i < m; ++i) Xm = fmaxf(Xm, s.pf[0][i][0]);
+#pragma unroll 1
+        for (int k = tid; k < NC; k += kT) {
+            const float4 r = row32<M>(s, k);
+            const float n2 = r.x * r.x + r.y * r.y + r.z * r.z;
+            if (!(n2 > kTiny && n2 < kHuge)) {
+                // a zero normal (a constant row) holds in its own cell; FP32 does not judge a tiny one
+                const bool zero = M == kDF ? n2 == 0.0f && s.rlo[4 * k] == 0.0f && s.rlo[4 * k + 1] == 0.0f && s.rlo[4 * k + 2] == 0.0f
+                                           : s.r64[4 * k] == 0.0 && s.r64[4 * k + 1] == 0.0 && s.r64[4 * k + 2] == 0.0;
+                if (!zero) s.si[4] = 1;
+                continue;
+            }
+            const float ri = rsqrtf(n2), rl1 = fabsf(r.x) + fabsf(r.y) + fabsf(r.z);
+            const float band = (float)a.delta * (n2 * ri) * 1.01f;     // delta |r|: the tolerance band
+            // the bound |r|_1 w_v + c_r: FP32 evaluation (4 terms), the row and the vertex rounded to FP32
+            // (8.5 u; 10.5 u with the row rounded towards zero), the vertex's and the row's own error
+            const float cr = M == kDF ? __fmaf_ru(s.err[k], Xm, __fmaf_ru(8.5f * kU, fabsf(r.w), band))
+                                      : __fmaf_ru(10.5f * kU, fabsf(r.w), band);
+            bool viol = false, edge = false;
+            int ea = s.pe[0][m - 1];
+#pragma unroll 2
+            for (int i = 0; i < m; ++i) {
+                const int eb = s.pe[0][i];
+                const bool own = k == ea || k == eb;
+                edge |= k == eb;
+                ea = eb;
+                if (own) continue;
+                const float4 V = *reinterpret_cast<const float4 *>(s.vf[i]);
+                const float sl = fmaf(r.x, V.x, fmaf(r.y, V.y, fmaf(r.z, V.z, r.w)));
+                const float B = __fmaf_ru(rl1, V.w, cr);
+                if (sl < -B) continue;
+                if (sl > B) { viol = true; continue; }
+                const int c = close_call<M>(a.max_n, a.delta, k, i, ri, rl1, band, Xm);
+                viol |= c == 1;
+                if (c == 2) s.si[4] = 1;
+            }
+            if (viol) {
+                if (edge) {
+                    s.si[4] = 1;                      // FP32 kept an edge that the vertices deny
+                } else {
+                    const int p = atomicAdd(s.si + 3, 1);
+                    s.viol[p] = k;
+                }
+            }
+        }
+        __syncthreads();
+        AM_TICK(tq0);
+        AM_PHASE(a, 5, tq1, tq0);
+        if (s.si[4]) return false;
+        const int nv = s.si[3];
+        if (nv == 0) {
+            *rounds = round;
+            return true;
+        }
+        if (round + 1 >= kFastFix || m + nv > kLines) return false;
+        // another round: the edges and the violated rows
+        if (tid < m) s.near_k[tid] = s.pe[0][tid];
+        else if (tid < m + nv) s.near_k[tid] = s.viol[tid - m];
+        n = m + nv;
+        __syncthreads();
+    }
+}
 
-    // box rows (exact), frame and the initial square (thread 0)
-    // (kDF: the pairs are stored as they are, exact FP32 words: the normal's components are
-    // 0 and +-1 and the offset is the host's split of the box, so no conversion runs here)
-    for (int i = tid; i < kBoxPlanes; i += kT) {
-        const int ax = i >> 1, k = N + i;
-        const float sg = (i & 1) ? -1.0f : 1.0f;
-        const float n0 = ax == 0 ? sg : 0.0f, n1 = ax == 1 ? sg : 0.0f, n2 = ax == 2 ? sg : 0.0f;
+// ------------------------------------------------------------------------------------------
+// one cell
+
+template <int M>
+__device__ __noinline__ void load_rows(const MarchArgs &a, int N, int64_t cell)
+{
+    const Sh s = make_sh(a.max_n);
+    const int tid = threadIdx.x;
+    // rows composed beforehand on the tensor cores, as FP32 pairs (the hi words [hi x 4] of
+    // rows 0..N, then their lo words [lo x 4])
+    // (signs as compose<M>, a_F last).  The pairs are the rows: the double-float tests are
+    // certified against them with no further row error, as FP64 tests take FP64 rows.
+    const float4 *src = reinterpret_cast<const float4 *>(a.rows_in) + (cell - a.begin) * (int64_t)(N + 1) * 2;
+    for (int k = tid; k < N; k += kT) {
+        const float4 h = __ldcs(src + k), l = __ldcs(src + (N + 1) + k);
         if (M == kFP64) {
             double *r = s.r64 + 4 * k;
-            r[0] = n0; r[1] = n1; r[2] = n2; r[3] = -a.box;
+            r[0] = (double)h.x + (double)l.x; r[1] = (double)h.y + (double)l.y;
+            r[2] = (double)h.z + (double)l.z; r[3] = (double)h.w + (double)l.w;
         } else {
-            *reinterpret_cast<float4 *>(s.rhi + 4 * k) = make_float4(n0, n1, n2, -a.box_hi);
-            *reinterpret_cast<float4 *>(s.rlo + 4 * k) = make_float4(0.0f, 0.0f, 0.0f, -a.box_lo);
+            *reinterpret_cast<float4 *>(s.rhi + 4 * k) = h;
+            *reinterpret_cast<float4 *>(s.rlo + 4 * k) = l;
             s.err[k] = 0.0f;
         }
     }
+    if (tid < 4) {
+        const float h = reinterpret_cast<const float *>(src + N)[tid];
+        const float l = reinterpret_cast<const float *>(src + 2 * N + 1)[tid];
+        s.aF[tid] = (double)h + (double)l;
+        if (M == kDF) { s.aFhi[tid] = h; s.aFlo[tid] = l; }
+    }
+    if (tid == 0) s.eF[0] = 0.0f;
+    __syncthreads();
+}
+
+// The sequential clip: the square about the box section cut by the candidate rows one by one, then
+// every row checked at every vertex; leaves the polygon in shared memory (s.si[0] vertices in buffer
+// s.si[1], status s.si[2]).  Returns the fix-up rounds, or -1 (kDF) when FP64 must decide the cell.
+// Out of line: the one-pass polygon (fast_face) takes nearly every cell.
+template <int M>
+__device__ __noinline__ int slow_clip(const MarchArgs &a, const NetDev &net, int64_t cell)
+{
+    const Sh s = make_sh(a.max_n);
+    const Arena &ar = a.ar;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int N = net.N, NC = N + kBoxPlanes;          // checked rows: neurons + box
+    int rounds = 0;
+    __syncthreads();
+    // the frame and the initial square (thread 0)
     if (tid == 0) {
         // an FP32 frame is enough: the square only has to contain the box section, and its
         // planes never bound a face (the box planes always cut them away)
@@ -978,7 +1608,7 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
         int loose = 0;
         for (int k = tid; k < N; k += kT) loose |= s.err[k] * s.rinv[k] > kDfLoose;
         if (tid == 0) loose |= s.eF[0] * rsqrtf((float)(s.aF[0] * s.aF[0] + s.aF[1] * s.aF[1] + s.aF[2] * s.aF[2])) > kDfLoose;
-        if (__syncthreads_or(loose)) return CellOut{0, 1};
+        if (__syncthreads_or(loose)) return -1;
     } else {
         __syncthreads();
     }
@@ -1028,7 +1658,6 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
     }
     __syncthreads();
 
-    AM_TICK(tp2);
     // ---- a4: warp 0 cuts the square with the candidates, nearest cutting row first.  A row
     // that holds on the polygon holds on every later (smaller) one, so it retires at once.
     if (wid == 0) {
@@ -1053,8 +1682,7 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
         // order-preserving unsigned image of the distance (scores may be negative)
         const unsigned du = __float_as_uint(d);
         const unsigned key = (du & 0x80000000u) ? ~du : (du | 0x80000000u);
-        AM_TICK(tp2a);
-        int m = s.si[0], buf = 0, status = 0, ncut = 0;
+            int m = s.si[0], buf = 0, status = 0, ncut = 0;
         const float aFf[4] = {s.aFhi[0], s.aFhi[1], s.aFhi[2], s.aFhi[3]};
         while (m > 0) {
             bool cut = false;
@@ -1085,21 +1713,18 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
             m = nm;
             ++ncut;
         }
-        AM_TICK(tp3a);
-        if (M == kDF && m > 0) df_final_vertices(s, m, buf, kVertexTol);
+            if (M == kDF && m > 0) df_final_vertices(s, m, buf, kVertexTol);
         if (lane == 0) { s.si[0] = m; s.si[1] = buf; s.si[2] = status; s.blk[6] += (unsigned long long)ncut; }
     }
     __syncthreads();
 
-    AM_TICK(tp3);
     // ---- a5: every row at every vertex; violators are cut in by warp 0 and the check repeats
-    int rounds = 0;
-    for (;; ++rounds) {
+    for (rounds = 0;; ++rounds) {
         const int m = s.si[0], buf = s.si[1];
-        if (M == kDF && s.si[10]) return CellOut{0, 1};     // a vertex too uncertain: FP64
+        if (M == kDF && s.si[10]) return -1;     // a vertex too uncertain: FP64
         // kDF: a polygon emptied (or a clip that failed) in the uncertified FP32 candidate pass
         // proves nothing: FP64 decides
-        if (M == kDF && (m == 0 || s.si[2])) return CellOut{0, 1};
+        if (M == kDF && (m == 0 || s.si[2])) return -1;
         if (m == 0 || s.si[2]) break;
         for (int i = tid; i < m; i += kT) {
             const double *v = s.pv[buf][i];
@@ -1171,7 +1796,7 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
         }
         if (tid == 0) s.si[5] = ndeg;
         __syncthreads();
-        if (s.si[4]) return CellOut{0, 1};
+        if (s.si[4]) return -1;
         const int nviol = s.si[3];
         if (nviol == 0) break;
         if (rounds + 1 >= kMaxFix) {
@@ -1201,29 +1826,113 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
         }
         __syncthreads();
     }
+    if (tid == 0) s.si[6] = 2;
+    __syncthreads();
+    return rounds;
+}
 
-    AM_TICK(tp4);
+// Warp 0: whether the polygon's area exceeds the smallest kept one, as a fan about vertex 0
+__device__ __noinline__ void area_test(int max_n, int buf, int m, double box)
+{
+    const Sh s = make_sh(max_n);
+    const int lane = threadIdx.x & 31;
+    const double *p0 = s.pv[buf][0];
+    double nx = 0.0, ny = 0.0, nz = 0.0;
+    for (int i = lane + 1; i < m - 1; i += 32) {
+        const double *p = s.pv[buf][i], *q = s.pv[buf][i + 1];
+        const double ax = p[0] - p0[0], ay = p[1] - p0[1], az = p[2] - p0[2];
+        const double bx = q[0] - p0[0], by = q[1] - p0[1], bz = q[2] - p0[2];
+        nx += ay * bz - az * by; ny += az * bx - ax * bz; nz += ax * by - ay * bx;
+    }
+    nx = warp_sum(nx); ny = warp_sum(ny); nz = warp_sum(nz);
+    const double amin = 2e-24 * box * box;          // twice the smallest kept area
+    if (lane == 0) s.si[6] = nx * nx + ny * ny + nz * nz > amin * amin;
+}
+
+// Pushes of keys wider than kThreadPushWords: one warp per edge, the key words split over the lanes
+__device__ __noinline__ void push_wide(const MarchArgs &a, int64_t cell, int buf, int m, int N, int pool0, int pool1, int pj)
+{
+    const Sh s = make_sh(a.max_n);
+    const Arena &ar = a.ar;
+    const unsigned long long h = *s.hsh;
+    for (int i = threadIdx.x >> 5; i < m; i += kNW) {
+        const int e = s.pe[buf][i];
+        if (e >= N) continue;
+        const double *p = s.pv[buf][i], *q = s.pv[buf][i + 1 == m ? 0 : i + 1];
+        const bool pool = e >= pool0 && e < pool1;
+        insert_neighbor_warp(ar, s.mask, cell, *s.nid, (unsigned)e, h ^ ar.zob[e] ^ (pool ? ar.zob[pool0 + pj] : 0ull),
+                             0.5f * (f32_toward_zero(p[0]) + f32_toward_zero(q[0])),
+                             0.5f * (f32_toward_zero(p[1]) + f32_toward_zero(q[1])),
+                             0.5f * (f32_toward_zero(p[2]) + f32_toward_zero(q[2])), true, pool0, pool1,
+                             pool ? pool0 + pj : -1);
+    }
+}
+
+struct CellOut {
+    int emit;        // corners written (0 = empty)
+    int ambiguous;   // kDF: an undecidable sign test; nothing written
+};
+
+template <int M>
+__device__ __forceinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net, int64_t cell)
+{
+    const Sh s = make_sh(a.max_n);
+    const Arena &ar = a.ar;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int N = s.hot->N;
+    long long tp0 = 0, tp1 = 0, tp2 = 0, tp3 = 0;
+    AM_TICK(tp0);
+    // box rows (exact)
+    // (kDF: the pairs are stored as they are, exact FP32 words: the normal's components are
+    // 0 and +-1 and the offset is the host's split of the box, so no conversion runs here)
+    if (tid < 4 * kBoxPlanes) {
+        const int i = tid >> 2, c = tid & 3;
+        const bool ax = c == (i >> 1);
+        if (M == kFP64) {
+            s.r64[4 * N + tid] = c == 3 ? -a.box : (ax ? ((i & 1) ? -1.0 : 1.0) : 0.0);
+        } else {
+            s.rhi[4 * N + tid] = c == 3 ? -a.box_hi : (ax ? ((i & 1) ? -1.0f : 1.0f) : 0.0f);
+            s.rlo[4 * N + tid] = c == 3 ? -a.box_lo : 0.0f;
+            s.err[N + i] = 0.0f;
+        }
+    }
+    if (tid < 11) s.si[tid] = 0;
+    int rounds = 0;
+    bool fast = false;
+    if (a.rows_in) {
+        load_rows<M>(a, N, cell);
+    } else {
+        compose<M>(net, s, false, a.max_n);
+        __syncthreads();
+        AM_TICK(tp1);
+        AM_PHASE(a, 0, tp0, tp1);
+        if (a.candidates == kCandNearest) {
+            fast = fast_face<M>(a, N, s, &rounds);
+            if (M == kDF && !fast) return CellOut{0, 1};
+        }
+    }
+    if (!fast) {
+        AM_TICK(tp2);
+        rounds = slow_clip<M>(a, net, cell);
+        AM_TICK(tp3);
+        AM_PHASE(a, 9, tp2, tp3);
+        if (rounds < 0) return CellOut{0, 1};
+    }
+
+    AM_TICK(tp2);
     // ---- a6 emit, a7 march
     const int m = s.si[0], buf = s.si[1];
     int status = s.si[2];
-    for (int i = 0; i < m; ++i)
-        if (s.pe[buf][i] >= N + kBoxPlanes) status = 3;   // a square edge: the plane misses the box
+    if (!fast)
+#pragma unroll 1
+        for (int i = 0; i < m; ++i)
+            if (s.pe[buf][i] >= N + kBoxPlanes) status = 3;   // a square edge: the plane misses the box
     int emit = (m >= 3 && status == 0) ? m : 0;
-    if (emit && wid == 0) {
-        // area of the polygon, as a fan about vertex 0 summed over the warp's lanes
-        const double *p0 = s.pv[buf][0];
-        double nx = 0.0, ny = 0.0, nz = 0.0;
-        for (int i = lane + 1; i < m - 1; i += 32) {
-            const double *p = s.pv[buf][i], *q = s.pv[buf][i + 1];
-            const double ax = p[0] - p0[0], ay = p[1] - p0[1], az = p[2] - p0[2];
-            const double bx = q[0] - p0[0], by = q[1] - p0[1], bz = q[2] - p0[2];
-            nx += ay * bz - az * by; ny += az * bx - ax * bz; nz += ax * by - ay * bx;
-        }
-        nx = warp_sum(nx); ny = warp_sum(ny); nz = warp_sum(nz);
-        const double amin = 2e-24 * a.box * a.box;          // twice the smallest kept area
-        if (lane == 0) s.si[6] = nx * nx + ny * ny + nz * nz > amin * amin;
+    if (emit && s.si[6] == 2) {
+        __syncthreads();
+        if (wid == 0) area_test(a.max_n, buf, m, a.box);
+        __syncthreads();
     }
-    __syncthreads();
     if (emit && !s.si[6]) emit = 0;
     if (emit > ar.maxv) {
         if (tid == 0) atomicOr(ar.counters + kStatus, kStFaceVerts);
@@ -1237,94 +1946,101 @@ __device__ __noinline__ CellOut solve_cell(const MarchArgs &a, const NetDev &net
         if (rounds) s.blk[3] += 1;
         if (status == 1 || status == 2) atomicOr(ar.counters + kStatus, kStClip);
     }
-    AM_TICK(tp4a);
+    AM_TICK(tp3);
+    AM_PHASE(a, 6, tp2, tp3);
     if (emit) {
-        for (int i = tid; i < m; i += kT) {
-            ar.edges[cell * ar.maxv + i] = s.pe[buf][i];
-            double *v = ar.verts + (cell * ar.maxv + i) * 3;
-            v[0] = s.pv[buf][i][0]; v[1] = s.pv[buf][i][1]; v[2] = s.pv[buf][i][2];
-        }
-        const unsigned long long h = __ldcg(ar.hash + cell);
-        const int nid = __ldcg(ar.net + cell);
+        // the face record (warps 1..; warp 0 pushes); m <= kMaxPoly
+        static_assert(3 * kMaxPoly + 32 <= kT && kMaxPoly + 32 <= kT, "one thread per word of a face");
+        if ((unsigned)(tid - 32) < 3u * (unsigned)m) ar.verts[cell * ar.maxv * 3 + (tid - 32)] = (&s.pv[buf][0][0])[tid - 32];
+        if ((unsigned)(tid - 32) < (unsigned)m) ar.edges[cell * ar.maxv + (tid - 32)] = s.pe[buf][tid - 32];
         // a max-pooled net (Sec. 5.2): crossing pooling plane n_units + i moves the pooled index j
         // to i (two key bits change), and the new cell enters through its pooling row of j
-        int pj = 0;
-        if (net.M >= 2)
-            for (int i = 0; i < net.M; ++i)
-                if (bit_of(s.mask, net.n_units + i)) { pj = i; break; }
-        const int pool0 = net.M >= 2 ? net.n_units : kNoPool, pool1 = net.M >= 2 ? N : kNoPool;
-        auto child = [&](int e, unsigned long long *hc, int *entry) {
-            if (e >= pool0 && e < pool1) {
-                *hc = h ^ ar.zob[e] ^ ar.zob[pool0 + pj];
-                *entry = pool0 + pj;
-            } else {
-                *hc = h ^ ar.zob[e];
-                *entry = -1;
-            }
-        };
+        int pj = 0, pool0 = kNoPool, pool1 = kNoPool;
+        if (s.hot->M >= 2) {
+            pool0 = s.hot->units;
+            pool1 = N;
+#pragma unroll 1
+            while (pj < s.hot->M - 1 && !bit_of(s.mask, pool0 + pj)) ++pj;
+        }
         if (ar.kw <= kThreadPushWords) {
-            // narrow keys: one thread per edge
-            for (int i = tid; i < m; i += kT) {
-                const int e = s.pe[buf][i];
-                if (e >= N) continue;
-                const double *p = s.pv[buf][i], *q = s.pv[buf][(i + 1) % m];
-                unsigned long long hc;
-                int entry;
-                child(e, &hc, &entry);
-                insert_neighbor(ar, s.mask, cell, nid, (unsigned)e, hc, (float)(0.5 * (p[0] + q[0])),
-                                (float)(0.5 * (p[1] + q[1])), (float)(0.5 * (p[2] + q[2])), pool0, pool1, entry);
+            // narrow keys: one lane of warp 0 per edge
+            if (wid == 0) {
+                const unsigned long long h = *s.hsh;
+                const int nid = *s.nid;
+#pragma unroll 1
+                for (int i0 = 0; i0 < m; i0 += 32) {
+                    const int i = i0 + lane, e = i < m ? s.pe[buf][i] : N;
+                    const bool on = e < N;
+                    unsigned long long hc = 0;
+                    int entry = -1;
+                    float mid[3] = {0.0f, 0.0f, 0.0f};
+                    if (on) {
+                        hc = h ^ (fast ? s.zb[i] : ar.zob[e]);
+                        if (e >= pool0 && e < pool1) {
+                            entry = pool0 + pj;
+                            hc ^= ar.zob[entry];
+                        }
+                        // the shared edge's midpoint: it only orders the neighbour's candidates
+                        const double *p = s.pv[buf][i], *q = s.pv[buf][i + 1 == m ? 0 : i + 1];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) mid[c] = 0.5f * (f32_toward_zero(p[c]) + f32_toward_zero(q[c]));
+                    }
+                    insert_neighbors(ar, s.mask, cell, nid, on, (unsigned)e, hc, mid[0], mid[1], mid[2], pool0, pool1, entry);
+                }
             }
         } else {
-            // wide keys: one warp per edge, the key words split over the lanes
-            for (int i = wid; i < m; i += kNW) {
-                const int e = s.pe[buf][i];
-                if (e >= N) continue;
-                const double *p = s.pv[buf][i], *q = s.pv[buf][(i + 1) % m];
-                unsigned long long hc;
-                int entry;
-                child(e, &hc, &entry);
-                insert_neighbor_warp(ar, s.mask, cell, nid, (unsigned)e, hc, (float)(0.5 * (p[0] + q[0])),
-                                     (float)(0.5 * (p[1] + q[1])), (float)(0.5 * (p[2] + q[2])), true, pool0,
-                                     pool1, entry);
-            }
+            push_wide(a, cell, buf, m, N, pool0, pool1, pj);
         }
     }
-    if (emit && tid < m) __threadfence();     // the face and the pushes of this thread
-    __syncthreads();
-    AM_TICK(tp5);
-    AM_PHASE(a, 0, tp0, tp1);
-    AM_PHASE(a, 1, tp1, tp2);
-    AM_PHASE(a, 2, tp2, tp2a);
-    AM_PHASE(a, 3, tp2a, tp3a);
-    AM_PHASE(a, 4, tp3a, tp3);
-    AM_PHASE(a, 5, tp3, tp4);
-    AM_PHASE(a, 6, tp4, tp4a);
-    AM_PHASE(a, 7, tp4a, tp5);
+    if (ar.kw > kThreadPushWords) __syncthreads();     // every warp has pushed
+    AM_TICK(tp2);
+    AM_PHASE(a, 7, tp3, tp2);
     return CellOut{emit, 0};
 }
 
+// FP64 for the cells (and nets) the double-float kernel does not decide
+__device__ __noinline__ void solve_cell_fp64(const MarchArgs &a, const NetDev &net, int64_t cell)
+{
+    solve_cell<kFP64>(a, net, cell);
+}
+
 template <int MODE>
-__device__ void process_cell(const MarchArgs &a, int64_t cell, const Sh &s)
+__device__ __forceinline__ void process_cell(const MarchArgs &a, int64_t cell, const Sh &s)
 {
     const Arena &ar = a.ar;
-    // the cell's record was written by another block of this launch: read it through L2
-    if (__ldcg(ar.nverts + cell) == -2) return;          // a duplicate seed id: never solved
-    const NetDev &net = a.nets[__ldcg(ar.net + cell)];
+    // the cell's record was written by another block of this launch: read it through L2, every
+    // word in flight at once
     const unsigned long long *key = ar.keys + cell * ar.kw;
-    for (int w = threadIdx.x; w < 2 * ar.kw; w += kT)       // all key words: pushes copy them
-        s.mask[w] = (unsigned)(__ldcg(key + (w >> 1)) >> ((w & 1) * 32));
+    const int dead = __ldcg(ar.nverts + cell), nid = __ldcg(ar.net + cell);
+    if ((int)threadIdx.x < 2 * ar.kw)                      // all key words (at most 256): pushes copy them
+        s.mask[threadIdx.x] = __ldcg(reinterpret_cast<const unsigned *>(key) + threadIdx.x);
+    if (threadIdx.x >= kT - 3) s.ent[kT - 1 - threadIdx.x] = __ldcg(ar.entry_pt + cell * 3 + (kT - 1 - threadIdx.x));
+    if (threadIdx.x == kT - 4) *s.hsh = __ldcg(ar.hash + cell);
+    if (threadIdx.x == kT - 5) *s.nid = nid;
+    const NetDev &net = a.nets[nid];
+    const bool other = s.hot->id != nid;
+    if (!other) {
+        if (MODE == kDF && s.hot->df_ok) touch_weights<kDF>(*s.hot);
+        else touch_weights<kFP64>(*s.hot);
+    }
     __syncthreads();
-    if (MODE == kDF && !net.df_ok && !a.rows_in) {
+    if (dead == -2) return;                              // a duplicate seed id: never solved
+    if (other) {
+        fill_hot(&net, nid, a.max_n);
+        __syncthreads();
+    }
+    if (MODE == kDF && !s.hot->df_ok && !a.rows_in) {
         if (threadIdx.x == 0) s.blk[4] += 1;             // solved in FP64 (the net's bound is too loose)
-        solve_cell<kFP64>(a, net, cell, s);
+        solve_cell_fp64(a, net, cell);
     } else if (MODE == kDF) {
-        const CellOut o = solve_cell<kDF>(a, net, cell, s);
+        const CellOut o = solve_cell<kDF>(a, net, cell);
         if (o.ambiguous) {
             if (threadIdx.x == 0) s.blk[4] += 1;
-            solve_cell<kFP64>(a, net, cell, s);
+            __syncthreads();
+            solve_cell_fp64(a, net, cell);
         }
     } else {
-        solve_cell<kFP64>(a, net, cell, s);
+        solve_cell<kFP64>(a, net, cell);
     }
 }
 
@@ -1345,42 +2061,41 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
     return v;
 }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p)
 {
     unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
 // Ticket of the next cell to solve, or -1 when the march is over (every handed-out cell is
 // finished), the ticket is beyond the limit, or a wait ran out of time (status flag set).
-// Waiting polls with plain acquire loads and an exponential back-off, so that idle blocks do
-// not flood the counters' cache lines with atomics.
+// Waiting polls the ticket's own flag with plain loads and an exponential back-off, so that idle
+// blocks do not flood the counters' cache lines with atomics.  An acquire empties the SM's L1, and with
+// it the weights of the block beside this one: the flag is read relaxed, with one fence once it is
+// set, and the counters (acquired: only they end the march) are read every 8th time.
 __device__ long long next_ticket(const MarchArgs &a)
 {
     unsigned long long *C = a.ar.counters;
     const long long t = (long long)atomicAdd(C + kHead, 1ull);
     if (t >= a.limit) return -1;
     const long long t0 = global_ns();
-    unsigned ns = 32;
+    unsigned ns = 16, poll = 0;
     for (;;) {
-        const unsigned long long n = ld_acquire(C + kNCells);
-        if ((unsigned long long)t < n) {
-            unsigned ns2 = 16;
-            while (ld_acquire(a.ar.ready + t) == 0u) {
-                if (global_ns() - t0 > a.wait_ns) { atomicOr(C + kStatus, kStTimeout); return -1; }
-                __nanosleep(ns2);
-                ns2 = min(2 * ns2, 256u);
-            }
+        if (ld_relaxed(a.ar.ready + t) != 0u) {
+            // acquire: the cell's record, written before its flag was released
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
             return t;
         }
-        // every handed-out cell finished (done read before the count: no cell can still push)
-        const unsigned long long done = ld_acquire(C + kDone);
-        const unsigned long long n2 = ld_acquire(C + kNCells);
-        if (done >= n2 && (unsigned long long)t >= n2) return -1;
-        if (global_ns() - t0 > a.wait_ns) { atomicOr(C + kStatus, kStTimeout); return -1; }
+        if ((poll++ & 7) == 7) {
+            // every handed-out cell finished (done read before the count: no cell can still push)
+            const unsigned long long done = ld_acquire(C + kDone);
+            const unsigned long long n = ld_acquire(C + kNCells);
+            if (done >= n && (unsigned long long)t >= n) return -1;
+            if (global_ns() - t0 > a.wait_ns) { atomicOr(C + kStatus, kStTimeout); return -1; }
+        }
         __nanosleep(ns);
-        ns = min(2 * ns, 256u);
+        ns = min(2 * ns, 128u);
     }
 }
 
@@ -1388,6 +2103,7 @@ __device__ long long next_ticket(const MarchArgs &a)
 __device__ __forceinline__ void blk_init(const Sh &s)
 {
     if (threadIdx.x < 8) s.blk[threadIdx.x] = 0ull;
+    if (threadIdx.x == 8) s.hot->id = -1;
     __syncthreads();
 }
 
@@ -1407,36 +2123,39 @@ __device__ __forceinline__ void blk_flush(const MarchArgs &a, const Sh &s)
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kT, AM_MIN_BLOCKS) march_persistent_kernel(MarchArgs a)
+__global__ void __launch_bounds__(kT, AM_MIN_BLOCKS) march_persistent_kernel(const __grid_constant__ MarchArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const Sh s = make_sh(smem, a.max_n, a.max_w);
+    const Sh s = make_sh(a.max_n);
     __shared__ long long ticket;
     blk_init(s);
     for (;;) {
         long long tw0 = 0, tw1 = 0;
         AM_TICK(tw0);
-        if (threadIdx.x == 0) ticket = next_ticket(a);
+        // the last warp draws the next ticket while warp 0 may still be pushing the last cell's
+        // neighbours
+        if (threadIdx.x == kT - 1) ticket = next_ticket(a);
         __syncthreads();
         AM_TICK(tw1);
         AM_PHASE(a, 8, tw0, tw1);
         const long long t = ticket;
         if (t < 0) break;
         process_cell<MODE>(a, t, s);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(a.ar.counters + kDone, 1ull);
+        if (threadIdx.x < 32) {
+            // the pushes of warp 0's lanes (kw > kThreadPushWords: of every warp, after a barrier) are
+            // counted before the cell is
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(a.ar.counters + kDone), "l"(1ull) : "memory");
+            }
         }
     }
     blk_flush(a, s);
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kT, AM_MIN_BLOCKS) march_range_kernel(MarchArgs a)
+__global__ void __launch_bounds__(kT, AM_MIN_BLOCKS) march_range_kernel(const __grid_constant__ MarchArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const Sh s = make_sh(smem, a.max_n, a.max_w);
+    const Sh s = make_sh(a.max_n);
     blk_init(s);
     if (a.list) {
         const int64_t n = (int64_t)__ldcg(a.list_count);
@@ -1455,18 +2174,19 @@ __global__ void __launch_bounds__(kT, AM_MIN_BLOCKS) march_range_kernel(MarchArg
 
 template <int MODE>
 __global__ void __launch_bounds__(kT, AM_MIN_BLOCKS)
-    compose_kernel(MarchArgs a, const NetDev *netp, const unsigned long long *keys, int kw_in, int64_t n,
+    compose_kernel(const __grid_constant__ MarchArgs a, const NetDev *netp, const unsigned long long *keys, int kw_in, int64_t n,
                    double *rows, float *err)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const Sh s = make_sh(smem, a.max_n, a.max_w);
+    const Sh s = make_sh(a.max_n);
     const NetDev &net = *netp;
     const int N = net.N, mw = 2 * ((a.max_n + 63) / 64);
+    fill_hot(netp, 0, a.max_n);
     for (int64_t c = blockIdx.x; c < n; c += gridDim.x) {
         for (int w = threadIdx.x; w < mw; w += kT)
             s.mask[w] = (w >> 1) < kw_in ? (unsigned)(keys[c * kw_in + (w >> 1)] >> ((w & 1) * 32)) : 0u;
         __syncthreads();
-        compose<MODE>(net, s, a.tc != 0, a.max_n + kBoxPlanes + kSquarePlanes);
+        compose<MODE>(net, s, a.tc != 0, a.max_n);
+        __syncthreads();
         double *out = rows + c * (int64_t)(N + 1) * 4;
         for (int k = threadIdx.x; k < N; k += kT) {
             double r[4];
