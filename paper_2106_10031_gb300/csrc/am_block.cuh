@@ -203,6 +203,83 @@ __device__ __forceinline__ void insert_neighbors(const Arena &ar, const unsigned
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ar.ready + id), "r"(1u) : "memory");
 }
 
+// The same pushes for the level schedule, any key width, plain nets: one neighbour per lane with `on` set.  The
+// lanes probe at once (the atomics of all edges are in flight together); a key to compare is read by the
+// whole warp, its words over the lanes, edge by edge.  The new cells are read only by later launches,
+// after this kernel has ended, so nothing is fenced.
+__device__ __forceinline__ void insert_neighbors_level(const Arena &ar, const unsigned *mask, int64_t parent, int net,
+                                                       bool on, unsigned flip, unsigned long long h, float px, float py,
+                                                       float pz)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const unsigned long long mine = slot_make(h, (unsigned long long)parent, flip);
+    unsigned long long pos = h & ar.slot_mask;
+    bool claimed = false, pending = on;
+    int probe = 0;
+#pragma unroll 1
+    while (__any_sync(full, pending) && probe < kMaxProbe) {
+        ++probe;
+        unsigned long long cur = 0ull;
+        if (pending) cur = atomicCAS(ar.slots + pos, 0ull, mine);
+        if (pending && cur == 0ull) { claimed = true; pending = false; }
+        unsigned cmp = __ballot_sync(full, pending && slot_tag(cur) == hash_tag(h));
+#pragma unroll 1
+        while (cmp) {
+            const int src = __ffs(cmp) - 1;
+            cmp &= cmp - 1;
+            const unsigned long long c = __shfl_sync(full, cur, src);
+            const unsigned fl = __shfl_sync(full, flip, src), fb = slot_flip(c);
+            const int64_t pb = slot_parent(c);
+            bool diff = lane == 0 && __ldcg(ar.net + pb) != net;
+#pragma unroll 1
+            for (int w = lane; w < 2 * ar.kw; w += 32) {
+                unsigned d = mask[w] ^ __ldcg(reinterpret_cast<const unsigned *>(ar.keys + pb * ar.kw) + w);
+                if ((int)(fl >> 5) == w) d ^= 1u << (fl & 31);
+                if (fb != kNoFlip && (int)(fb >> 5) == w) d ^= 1u << (fb & 31);
+                diff |= d != 0u;
+            }
+            diff = __any_sync(full, diff);
+            if (lane == src && !diff) pending = false;        // seen before
+        }
+        pos = (pos + 1) & ar.slot_mask;
+    }
+    if (pending) atomicOr(ar.counters + kStatus, kStHashFull);
+    unsigned who = __ballot_sync(full, claimed);
+    if (who == 0u) return;
+    const int lead = __ffs(who) - 1;
+    unsigned long long base = 0ull;
+    if (lane == lead) base = atomicAdd(ar.counters + kNCells, (unsigned long long)__popc(who));
+    base = __shfl_sync(full, base, lead);
+    const long long id = (long long)base + __popc(who & ((1u << lane) - 1u));
+    if (claimed) {
+        if (id >= ar.cap) {
+            atomicOr(ar.counters + kStatus, kStCellCap);
+        } else {
+            ar.net[id] = net;
+            ar.hash[id] = h;
+            ar.nverts[id] = -1;
+            ar.entry_plane[id] = (int32_t)flip;
+            ar.parent[id] = (int32_t)parent;
+            ar.entry_pt[id * 3 + 0] = px;
+            ar.entry_pt[id * 3 + 1] = py;
+            ar.entry_pt[id * 3 + 2] = pz;
+            ar.ready[id] = 1u;
+        }
+    }
+#pragma unroll 1
+    while (who) {
+        const int src = __ffs(who) - 1;
+        who &= who - 1;
+        const long long nid = __shfl_sync(full, id, src);
+        const unsigned fl = __shfl_sync(full, flip, src);
+        if (nid >= ar.cap) continue;
+        unsigned *kn = reinterpret_cast<unsigned *>(ar.keys + nid * ar.kw);
+#pragma unroll 1
+        for (int w = lane; w < 2 * ar.kw; w += 32) kn[w] = mask[w] ^ ((int)(fl >> 5) == w ? 1u << (fl & 31) : 0u);
+    }
+}
+
 // The same push by a whole warp (every lane calls it with the same arguments): lane 0 claims
 // the slot and the id, the lanes copy and compare the key words in parallel.  For wide keys
 // (N = 4096: 64 words) this turns 2 kw serial L2 round trips per tag hit into 2 kw / 32.

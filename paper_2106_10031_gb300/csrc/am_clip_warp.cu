@@ -9,11 +9,12 @@
 //   candidates : each lane keeps the two rows nearest to the point the cell was entered through
 //                among the rows it scans, and with learned candidates also the row the proposal
 //                scores highest among them (the proposal extends the nearest set);
-//   clip       : the square about the box section is cut by those 64 (96) candidates, nearest cutting
-//                row first, in FP32 (Eq. 11 per new vertex), then every vertex is re-solved in
-//                FP64 from its two planes;
-//   check      : every row at every vertex with a certified FP32 bound; close calls in FP64;
-//                violated rows are cut in (FP64) and the check repeats;
+//   clip       : a square about the box section, in FP32 coordinates of the face plane, is cut by the
+//                lines of those 64 (96) candidates, nearest cutting line first, then every vertex
+//                is solved in FP64 from its two planes (Eq. 11);
+//   check      : every row at every vertex with a certified FP32 bound; the rows it does not clear
+//                (the edges' own among them) one by one, close calls in FP64; violated rows join
+//                the edges as the lines of another round;
 //   emit, push : the face record, then each neuron edge pushes its neighbour (Alg. 1 step 10).
 // A cell that needs more than this (a test the FP64 close call cannot decide, a row within the
 // tolerance band of a vertex, a polygon beyond the warp's capacity, too many violators) is
@@ -428,20 +429,195 @@ __device__ bool wemit(const MarchArgs &a, WarpSh &S, int64_t cell, int net_id, i
 
 }  // namespace
 
-int clip_warp_smem_bytes() { return warp_smem_bytes(); }
-
 #ifndef AM_CLIP_MIN_BLOCKS
 #define AM_CLIP_MIN_BLOCKS 3
 #endif
-__global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel(MarchArgs a)
+// ---- the clip of a level
+//
+// What bounds it is instruction issue and fetch: 24 warps per SM run different cells through different parts
+// of the code, and above 32 KB of it an SM sub-partition fetches one instruction every two cycles (above
+// 128 KB, one every six).  So the code is short (40 KB, 141 before), its loops rolled, and the work per
+// (row, vertex) pair is four FMAs and a maximum.  The polygon lives in the warp's registers, one vertex
+// per lane, and the pushes of all edges probe the hash table at once.  Per mesh: 3-[256]x8-1 (1.63 M
+// faces, learned candidates) 71.5 -> 33.3 ms, a decoder (3+256)-[128]x8-1 (884,000 faces) 29.2 -> 12.3 ms,
+// 3-[60]x6-1 (72,000 faces) 2.6 -> 1.3 ms.  The rows read twice are 32.8 KB of hi words per cell at N = 2048:
+// 107 GB of the first mesh, 16 ms at the measured copy bandwidth.
+
+constexpr int kRing = 32;         // polygon vertices: one per lane
+constexpr int kFlag = 64;         // rows per check that the maximum test may hand to the exact one
+
+struct ClipSh {
+    double pv[kRing][3];          // FP64 vertices
+    double e64[kRing][4];         // the edges' rows in FP64
+    float4 vf[kRing];             // FP32 vertices and the vertex term of the check's bound
+    int pe[kRing];                // edge planes (edge i: vertex i -> i + 1)
+    int flag[kFlag];              // rows of the exact test
+    int viol[32];                 // violated rows
+    int nflag, nviol;
+    double aF[4];
+    unsigned key[2 * kWMaxKw];    // the cell's key as 32-bit words (pushes copy it)
+};
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// hi words of row k: memory, or a box row
+__device__ __forceinline__ float4 clip_row(const float4 *p, int N, float box, int k)
+{
+    if (k < N) return __ldg(p + k);
+    const int i = k - N;
+    const float sg = (i & 1) ? -1.0f : 1.0f;
+    return make_float4((i >> 1) == 0 ? sg : 0.0f, (i >> 1) == 1 ? sg : 0.0f, (i >> 1) == 2 ? sg : 0.0f, -box);
+}
+
+// The face plane's frame about the entry point e: coordinates (u . (x - e), w . (x - e)).  line: row r there
+// as a unit normal and an offset, (0, 0, -1) when it is (nearly) parallel to the plane.
+struct PlaneFrame {
+    float u0, u1, u2, w0, w1, w2, ex, ey, ez;
+    __device__ __forceinline__ void set(float f0, float f1, float f2)
+    {
+        const float inv = rsqrtf(f0 * f0 + f1 * f1 + f2 * f2);
+        const float n0 = f0 * inv, n1 = f1 * inv, n2 = f2 * inv;
+        const float ax = fabsf(n0), ay = fabsf(n1), az = fabsf(n2);
+        const int ei = (ax <= ay && ax <= az) ? 0 : (ay <= az ? 1 : 2);
+        u0 = ei == 0 ? 0.0f : (ei == 1 ? -n2 : n1);       // u = n x e_i, w = n x u
+        u1 = ei == 0 ? n2 : (ei == 1 ? 0.0f : -n0);
+        u2 = ei == 0 ? -n1 : (ei == 1 ? n0 : 0.0f);
+        const float un = rsqrtf(u0 * u0 + u1 * u1 + u2 * u2);
+        u0 *= un; u1 *= un; u2 *= un;
+        w0 = n1 * u2 - n2 * u1; w1 = n2 * u0 - n0 * u2; w2 = n0 * u1 - n1 * u0;
+    }
+    __device__ __forceinline__ float3 line(const float4 r) const
+    {
+        const float A = r.x * u0 + r.y * u1 + r.z * u2, B = r.x * w0 + r.y * w1 + r.z * w2, q2 = A * A + B * B;
+        const bool on = q2 > 1e-10f * (r.x * r.x + r.y * r.y + r.z * r.z);
+        const float q = on ? rsqrt_approx(q2) : 0.0f;
+        return make_float3(A * q, B * q, on ? fmaf(r.x, ex, fmaf(r.y, ey, fmaf(r.z, ez, r.w))) * q : -1.0f);
+    }
+};
+
+// One row of the exact test: its FP32 value against the bound at every vertex that is not its own, close
+// calls in FP64 from the exact pair.  Returns 1 when violated, 2 when FP64 cannot decide or it is an
+// edge that is violated elsewhere, 0 when it holds; *close counts the FP64 evaluations.  Out of line:
+// a cell has it for its edges' rows and one row in a few cells.
+__device__ __noinline__ int clip_exact_row(ClipSh &S, const float4 *p, int N, float box, float box_lo, int k, int m,
+                                           float delta, int *close)
+{
+    const float4 r = clip_row(p, N, box, k);
+    const float rl1 = fabsf(r.x) + fabsf(r.y) + fabsf(r.z);
+    const float band = delta * sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);      // delta |r|: the tolerance band
+    const float cr = __fmaf_ru(8.5f * kWU, fabsf(r.w), band);
+    bool viol = false, amb = false, edge = false;
+    int ea = S.pe[m - 1];
+#pragma unroll 1
+    for (int i = 0; i < m; ++i) {
+        const int eb = S.pe[i];
+        const bool own = k == ea || k == eb;
+        edge |= k == eb;
+        ea = eb;
+        if (own) continue;
+        const float4 V = S.vf[i];
+        const float sl = fmaf(r.x, V.x, fmaf(r.y, V.y, fmaf(r.z, V.z, r.w)));
+        const float B = __fmaf_ru(rl1, V.w, cr);
+        if (sl < -B) continue;
+        if (sl > B) { viol = true; continue; }
+        ++*close;
+        const float4 l = k < N ? __ldg(p + (N + 1) + k) : make_float4(0.0f, 0.0f, 0.0f, -box_lo);
+        const double r0 = (double)r.x + (double)l.x, r1 = (double)r.y + (double)l.y, r2 = (double)r.z + (double)l.z,
+                     r3 = (double)r.w + (double)l.w;
+        const double *v6 = S.pv[i];
+        const double s6 = r0 * v6[0] + r1 * v6[1] + r2 * v6[2] + r3;
+        const double m6 = fabs(r0 * v6[0]) + fabs(r1 * v6[1]) + fabs(r2 * v6[2]) + fabs(r3);
+        const float X = fmaxf(1.0f, fmaxf(fabsf(V.x), fmaxf(fabsf(V.y), fabsf(V.z)))) * 1.0001f;
+        const double B6 = (double)rl1 * 1.0001 * (double)(4e-16f * X * 1.01f) + (double)band + 1e-15 * m6;
+        if (s6 > B6) viol = true;
+        else if (!(s6 < -B6)) amb = true;
+    }
+    return amb || (viol && edge) ? 2 : (viol ? 1 : 0);
+}
+
+// whether the FP64 polygon's area exceeds the smallest kept one (a fan about vertex 0 summed over the
+// lanes); out of line: FP32 decides all but degenerate faces
+__device__ __noinline__ bool clip_area(const ClipSh &S, int m, double box)
+{
+    const int lane = threadIdx.x & 31;
+    const double *p0 = S.pv[0];
+    double nx = 0.0, ny = 0.0, nz = 0.0;
+    if (lane >= 1 && lane < m - 1) {
+        const double *p = S.pv[lane], *q = S.pv[lane + 1];
+        const double ax = p[0] - p0[0], ay = p[1] - p0[1], az = p[2] - p0[2];
+        const double bx = q[0] - p0[0], by = q[1] - p0[1], bz = q[2] - p0[2];
+        nx = ay * bz - az * by; ny = az * bx - ax * bz; nz = ax * by - ay * bx;
+    }
+    nx = warp_sum(nx); ny = warp_sum(ny); nz = warp_sum(nz);
+    const double amin = 2e-24 * box * box;            // twice the smallest kept area
+    return nx * nx + ny * ny + nz * nz > amin * amin;
+}
+
+// The ring's vertices in FP64 from its planes' exact pairs (Eq. 11, solve3's Cramer's rule): the rows as
+// FP64 one lane per coefficient, the vertices one lane per coordinate (an FP64 warp instruction takes
+// about 64 cycles for one lane as for 32: 25 of them per face instead of 110).  Also the FP32 vertices and
+// the vertex term w = 8.5 u X + the vertex's own error of the check's bound.  False: a vertex is not finite.
+__device__ __forceinline__ bool clip_vertices(ClipSh &S, const float4 *p, int N, float box, float box_lo, int m)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned FULL = 0xffffffffu;
+    const float *pf = reinterpret_cast<const float *>(p);
+#pragma unroll 1
+    for (int q = lane; q < 4 * m; q += 32) {
+        const int k = S.pe[q >> 2], c = q & 3, i = k - N;
+        float h, l;
+        if (k < N) {
+            h = __ldg(pf + 4 * k + c);
+            l = __ldg(pf + 4 * (N + 1 + k) + c);
+        } else {
+            h = c == 3 ? -box : (c == (i >> 1) ? ((i & 1) ? -1.0f : 1.0f) : 0.0f);
+            l = c == 3 ? -box_lo : 0.0f;
+        }
+        S.e64[q >> 2][c] = (double)h + (double)l;
+    }
+    __syncwarp();
+    const int v = lane / 3, d = lane - 3 * v, d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+    const int l0 = 3 * v, l1 = l0 + 1, l2 = min(l0 + 2, 31);
+    bool good = true;
+#pragma unroll 1
+    for (int b = 0; b < m; b += 10) {
+        const int i = b + v;
+        const bool on = v < 10 && i < m;
+        const int iq = on ? i : 0, ip = iq == 0 ? m - 1 : iq - 1;
+        const double *pa = S.e64[ip], *q = S.e64[iq], *f = S.aF;
+        const double c0 = q[d1] * f[d2] - q[d2] * f[d1], c1 = f[d1] * pa[d2] - f[d2] * pa[d1],
+                     c2 = pa[d1] * q[d2] - pa[d2] * q[d1];
+        const double det = pa[0] * __shfl_sync(FULL, c0, l0) + pa[1] * __shfl_sync(FULL, c0, l1) + pa[2] * __shfl_sync(FULL, c0, l2);
+        const double inv = -1.0 / det;
+        const double x = (pa[3] * c0 + q[3] * c1 + f[3] * c2) * inv;
+        const float xf = (float)x;
+        float X = fmaxf(1.0f, fabsf(xf));
+        X = fmaxf(X, fmaxf(__shfl_sync(FULL, X, l0), fmaxf(__shfl_sync(FULL, X, l1), __shfl_sync(FULL, X, l2)))) * 1.0001f;
+        if (on) {
+            S.pv[i][d] = x;
+            reinterpret_cast<float *>(S.vf + i)[d] = xf;
+            if (d == 0) S.vf[i].w = __fmaf_ru(8.5f * kWU, X, 4e-16f * X * 1.01f);
+            good = good && isfinite(xf);
+        }
+    }
+    return __all_sync(FULL, good);
+}
+
+__global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ __align__(16) unsigned char wsm[];
-    WarpSh &S = reinterpret_cast<WarpSh *>(wsm)[threadIdx.x >> 5];
+    ClipSh &S = reinterpret_cast<ClipSh *>(wsm)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     const Arena &ar = a.ar;
-    unsigned long long n_solved = 0, n_empty = 0, n_fix = 0, n_cuts = 0, n_close = 0, n_fb = 0;
+    unsigned n_solved = 0, n_empty = 0, n_fix = 0, n_cuts = 0, n_close = 0, n_fb = 0;
     const int64_t stride = (int64_t)gridDim.x * kWW;
+    const float box = a.box_hi, delta = (float)a.delta * 1.01f;
     // with a.work the warps take cells one at a time from a shared counter (cells differ in
     // their cost: the cuts, the fix-up rounds), else in a fixed stride
     auto next = [&](int64_t cur) -> int64_t {
@@ -455,141 +631,279 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
         if (__ldcg(ar.nverts + cell) == -2) continue;          // a duplicate seed id: never solved
         const int net_id = __ldcg(ar.net + cell);
         const int N = a.nets[net_id].N;
-        WRows rv;
-        int m = wcell_setup(a, S, cell, N, rv);
-        bool fallback = m == 0;
-        // ---- candidates: per lane the two best of the rows it scans
-        const float px = __ldcg(ar.entry_pt + cell * 3), py = __ldcg(ar.entry_pt + cell * 3 + 1),
-                    pz = __ldcg(ar.entry_pt + cell * 3 + 2);
-        const int entry = __ldcg(ar.entry_plane + cell);
+        const float4 *p = reinterpret_cast<const float4 *>(a.rows_in) + (cell - a.begin) * 2 * (int64_t)(N + 1);
+        PlaneFrame fr;
+        fr.ex = __ldcg(ar.entry_pt + cell * 3); fr.ey = __ldcg(ar.entry_pt + cell * 3 + 1);
+        fr.ez = __ldcg(ar.entry_pt + cell * 3 + 2);
+        __syncwarp();                                    // the last cell's readers of S are done
+#pragma unroll 1
+        for (int w = lane; w < 2 * ar.kw; w += 32) S.key[w] = __ldcg(reinterpret_cast<const unsigned *>(ar.keys + cell * ar.kw) + w);
+        if (lane < 4) S.aF[lane] = (double)reinterpret_cast<const float *>(p + N)[lane] + (double)reinterpret_cast<const float *>(p + 2 * N + 1)[lane];
+        const float4 F = __ldg(p + N);
         const bool learned = a.candidates == kCandLearned && a.scores_in && a.prop.n_out == N;
         const __nv_bfloat16 *sc = learned ? a.scores_in + (cell - a.begin) * (int64_t)a.scores_ld : nullptr;
-        float b1 = 3.0e38f, b2 = 3.0e38f, b3 = 3.0e38f, s3 = 3.0e38f;
-        int k1 = -1, k2 = -1, k3 = -1;
-        if (!fallback) {
-            auto consider = [&](int k, const float4 r, float score) {
-                const float n2 = r.x * r.x + r.y * r.y + r.z * r.z;
-                if (n2 == 0.0f) return;
-                const float d = fabsf(r.x * px + r.y * py + r.z * pz + r.w) * rsqrtf(n2);
-                if (d < b1) { b2 = b1; k2 = k1; b1 = d; k1 = k; }
-                else if (d < b2) { b2 = d; k2 = k; }
-                if (learned && k < N) {
-                    // the learned proposal adds the row it scores highest among this lane's
-                    const float q = k == entry ? -3.0e37f : -score;
-                    if (q < s3) { s3 = q; k3 = k; b3 = d; }
-                }
-            };
-            // the neuron rows and their scores, 8 of each in flight per lane; then the box rows
-            // (lanes 0..5)
-            for (int k0 = lane; k0 < N; k0 += 32 * 8) {
-                float4 r[8];
-                float q[8];
+        // ---- candidates: per lane the two rows nearest to the entry point of those it scans, by the
+        //      distance's bits with the scan's index (N <= 8192: below 256) in the lowest eight
+        unsigned b1 = 0xffffffffu, b2 = 0xffffffffu;
+        float s3 = 3.0e38f;
+        int k3 = -1;
+#pragma unroll 1
+        for (int u0 = 0; 32 * u0 < N; u0 += 8) {
+            float4 r[8];
+            float q[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k = lane + 32 * (u0 + u);
+                r[u] = k < N ? __ldg(p + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+            if (learned) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const int k = k0 + 32 * u;
-                    r[u] = k < N ? __ldg(rv.p + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    q[u] = learned && k < N ? __bfloat162float(sc[k]) : 0.0f;
+                    const int k = lane + 32 * (u0 + u);
+                    q[u] = k < N ? -__bfloat162float(sc[k]) : 3.0e38f;
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
-                    if (k0 + 32 * u < N) consider(k0 + 32 * u, r[u], q[u]);
+                    if (q[u] < s3) { s3 = q[u]; k3 = lane + 32 * (u0 + u); }
             }
-            if (lane < kBoxPlanes) consider(N + lane, rv.hi(N + lane), 0.0f);
-            if (k3 == k1 || k3 == k2) k3 = -1;            // already a candidate
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float n2 = r[u].x * r[u].x + r[u].y * r[u].y + r[u].z * r[u].z;
+                const float d = fabsf(fmaf(r[u].x, fr.ex, fmaf(r[u].y, fr.ey, fmaf(r[u].z, fr.ez, r[u].w)))) * rsqrt_approx(n2);
+                // no normal (or no row): infinity or not a number, above every distance
+                const unsigned c = n2 > 0.0f ? (__float_as_uint(d) & ~255u) | (unsigned)(u0 + u) : 0xffffffffu;
+                b2 = min(b2, max(b1, c));
+                b1 = min(b1, c);
+            }
         }
-        // ---- the candidate clip (FP32): nearest cutting row first; a row that holds on the
-        //      polygon holds on every later (smaller) one and retires
-        int buf = 0, ncut = 0;
-        {
-            // up to three candidate slots per lane, cut nearest first (the learned slot too)
-            const int kk[3] = {k1, k2, k3};
-            const unsigned key[3] = {order_key(b1), order_key(b2), order_key(b3)};
-            bool live[3] = {k1 >= 0, k2 >= 0, k3 >= 0};
-            float cr[3][4], cri[3];
+        // slots: the nearest two (a box row in the place of the second where it is nearer) and the
+        // proposal's best row
+        int kk[3] = {b1 == 0xffffffffu ? -1 : lane + 32 * (int)(b1 & 255u), b2 == 0xffffffffu ? -1 : lane + 32 * (int)(b2 & 255u),
+                     learned ? k3 : -1};
+        if (lane < kBoxPlanes) {
+            const float4 r = clip_row(p, N, box, N + lane);
+            const float d = fabsf(fmaf(r.x, fr.ex, fmaf(r.y, fr.ey, fmaf(r.z, fr.ez, r.w))));
+            if (kk[1] < 0 || __float_as_uint(d) < b2) kk[1] = N + lane;
+        }
+        if (kk[2] == kk[0] || kk[2] == kk[1]) kk[2] = -1;      // already a candidate
+        fr.set(F.x, F.y, F.z);
+        const float nn = F.x * F.x + F.y * F.y + F.z * F.z;
+        bool fallback = !(nn > 0.0f && isfinite(nn));
+        int m = 0, rounds = 0, close = 0;
+        unsigned ncut = 0;
+        float vx = 0.0f, vy = 0.0f;
+        while (!fallback) {
+            // ---- the candidate clip (FP32, in the plane): a square about the box section, then the nearest
+            //      cutting line first; a line that holds on the polygon holds on every smaller one and retires
+            float cA[3], cB[3], cC[3];
+            bool live[3];
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                if (kk[j] >= 0) rv.f32(kk[j], cr[j]);
-                else cr[j][0] = cr[j][1] = cr[j][2] = cr[j][3] = 0.0f;
-                cri[j] = kk[j] >= 0 ? rsqrtf(cr[j][0] * cr[j][0] + cr[j][1] * cr[j][1] + cr[j][2] * cr[j][2]) : 0.0f;
+                float3 L = make_float3(0.0f, 0.0f, -1.0f);
+                if (kk[j] >= 0) L = fr.line(clip_row(p, N, box, kk[j]));
+                cA[j] = L.x; cB[j] = L.y; cC[j] = L.z;
+                live[j] = kk[j] >= 0;
             }
-            while (!fallback && m > 0) {
-                bool c[3] = {false, false, false};
+            const float sz = 2.1f * 1.7320508f * box;    // the entry point lies in the box
+            vx = (lane == 1 || lane == 2) ? sz : -sz;
+            vy = lane >= 2 ? sz : -sz;
+            float eA = lane == 1 ? 1.0f : (lane == 3 ? -1.0f : 0.0f), eB = lane == 0 ? -1.0f : (lane == 2 ? 1.0f : 0.0f), eC = -sz;
+            int id = -1 - lane;                          // the square's edges: never the face's
+            m = 4;
+#pragma unroll 1
+            while (true) {
+                float mx[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
+#pragma unroll 1
+                for (int i = 0; i < m; ++i) {
+                    const float x = __shfl_sync(FULL, vx, i), y = __shfl_sync(FULL, vy, i);
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) mx[j] = fmaxf(mx[j], fmaf(cA[j], x, fmaf(cB[j], y, cC[j])));
+                }
+                unsigned mine = 0xffffffffu;
+                int slot = 0;
 #pragma unroll
                 for (int j = 0; j < 3; ++j) {
-                    if (!live[j]) continue;
-                    for (int i = 0; i < m && !c[j]; ++i) c[j] = wpdist(cr[j], cri[j], S.pf[buf][i]) > 1e-7f;
+                    live[j] = live[j] && mx[j] > 1e-7f;
+                    const unsigned c = live[j] ? __float_as_uint(fabsf(cC[j])) : 0xffffffffu;
+                    if (c < mine) { mine = c; slot = j; }
                 }
-#pragma unroll
-                for (int j = 0; j < 3; ++j) live[j] = c[j];
-                if (!__any_sync(FULL, c[0] || c[1] || c[2])) break;
-                unsigned mine = 0xffffffffu;
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (c[j]) mine = min(mine, key[j]);
-                const unsigned kmin = __reduce_min_sync(FULL, mine);
-                unsigned cand = 0xffffffffu;
+                const unsigned best = __reduce_min_sync(FULL, mine);
+                if (best == 0xffffffffu) break;
+                const int src = __ffs(__ballot_sync(FULL, mine == best)) - 1;
+                const float A = __shfl_sync(FULL, slot == 0 ? cA[0] : (slot == 1 ? cA[1] : cA[2]), src);
+                const float B = __shfl_sync(FULL, slot == 0 ? cB[0] : (slot == 1 ? cB[1] : cB[2]), src);
+                const float C = __shfl_sync(FULL, slot == 0 ? cC[0] : (slot == 1 ? cC[1] : cC[2]), src);
+                const int kc = __shfl_sync(FULL, slot == 0 ? kk[0] : (slot == 1 ? kk[1] : kk[2]), src);
 #pragma unroll
                 for (int j = 0; j < 3; ++j)
-                    if (c[j] && key[j] == kmin) cand = min(cand, (unsigned)kk[j]);
-                const int kc = (int)__reduce_min_sync(FULL, cand);
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (kk[j] == kc) live[j] = false;
-                bool sw;
-                const int nm = wcut<float>(S, S.pf, m, buf, kc, 1e-7f, S.aFhi, rv, &sw);
-                if (nm < 0) { fallback = true; break; }
-                if (sw) buf ^= 1;
-                m = nm;
+                    if (lane == src && slot == j) live[j] = false;
+                // the cut: the vertices beyond the line leave, two on it take their place
+                const unsigned full = m == 32 ? FULL : (1u << m) - 1u;
+                const unsigned out = __ballot_sync(FULL, lane < m && fmaf(A, vx, fmaf(B, vy, C)) > 1e-7f);
+                const int nout = __popc(out);
+                const unsigned first = out & ~((out << 1) | (out >> (m - 1))) & full;
+                const int nin = m - nout;
+                // nothing cut (rounding), or everything, or more than one run, or no lane left
+                if (nout == 0) continue;
+                if (nin == 0 || __popc(first) != 1 || nin + 2 > kRing) { fallback = true; break; }
+                const int ia = __ffs(first) - 1;
+                int ib = ia + nout - 1;
+                if (ib >= m) ib -= m;
+                // lane q takes the q-th kept vertex after the run; then the run's two ends with their edges
+                int from = ib + 1 + lane;
+                if (from >= m) from -= m;
+                if (lane == nin) from = ia == 0 ? m - 1 : ia - 1;
+                if (lane == nin + 1) from = ib;
+                from &= 31;
+                vx = __shfl_sync(FULL, vx, from); vy = __shfl_sync(FULL, vy, from);
+                eA = __shfl_sync(FULL, eA, from); eB = __shfl_sync(FULL, eB, from); eC = __shfl_sync(FULL, eC, from);
+                id = __shfl_sync(FULL, id, from);
+                if (lane == nin || lane == nin + 1) {
+                    const float D = __fdividef(1.0f, eA * B - eB * A);
+                    vx = (eB * C - B * eC) * D;
+                    vy = (A * eC - eA * C) * D;
+                    if (lane == nin) { eA = A; eB = B; eC = C; id = kc; }
+                }
+                m = nin + 2;
                 ++ncut;
             }
+            if (fallback) break;
+            // a square's edge left (an open polygon), or one that FP32 emptied, proves nothing
+            if (__any_sync(FULL, lane < m && (id < 0 || !isfinite(vx) || !isfinite(vy)))) { fallback = true; break; }
+            if (lane < m) S.pe[lane] = id;
+            if (lane == 0) S.nflag = S.nviol = 0;
+            __syncwarp();
+            if (!clip_vertices(S, p, N, box, a.box_lo, m)) { fallback = true; break; }
+            __syncwarp();
+            if (a.chk && m <= kChkMaxV) break;           // the dense check runs on the tensor cores (check_tc)
+            // ---- the all-row check: per row the largest of its value plus its bound over the vertices (the
+            //      bound |r|_1 w + c_r with c_r = 11 u |r_3| + delta |r|_1: rounding of the sum included);
+            //      below zero the row holds everywhere, else the exact test takes it
+#pragma unroll 1
+            for (int k0 = lane; k0 < N; k0 += 32 * 4) {
+                float4 r[4];
+                float l1[4], c0[4], mx[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = k0 + 32 * u;
+                    r[u] = k < N ? __ldg(p + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    l1[u] = (fabsf(r[u].x) + fabsf(r[u].y) + fabsf(r[u].z)) * 1.3f;
+                    // a zero normal (a constant row, which holds in its own cell) or no row
+                    c0[u] = l1[u] > 0.0f ? r[u].w + fmaf(11.0f * kWU, fabsf(r[u].w), delta * l1[u]) : -3.0e38f;
+                    mx[u] = -3.0e38f;
+                }
+#pragma unroll 1
+                for (int i = 0; i < m; ++i) {
+                    const float4 V = S.vf[i];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        mx[u] = fmaxf(mx[u], fmaf(r[u].x, V.x, fmaf(r[u].y, V.y, fmaf(r[u].z, V.z, fmaf(l1[u], V.w, c0[u])))));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (!(mx[u] < 0.0f)) {
+                        const int q = atomicAdd(&S.nflag, 1);
+                        if (q < kFlag) S.flag[q] = k0 + 32 * u;
+                    }
+            }
+            if (lane < kBoxPlanes) {                     // the box's rows: coordinate +-x, y, z against the box
+                float mx = -3.0e38f;
+#pragma unroll 1
+                for (int i = 0; i < m; ++i) {
+                    const float x = reinterpret_cast<const float *>(S.vf + i)[lane >> 1], w = S.vf[i].w;
+                    mx = fmaxf(mx, ((lane & 1) ? -x : x) - box + fmaf(1.3f, w, 11.0f * kWU * box + delta));
+                }
+                if (!(mx < 0.0f)) {
+                    const int q = atomicAdd(&S.nflag, 1);
+                    if (q < kFlag) S.flag[q] = N + lane;
+                }
+            }
+            __syncwarp();
+            const int nf = S.nflag;
+            bool amb = nf > kFlag;
+#pragma unroll 1
+            for (int t = lane; t < min(nf, kFlag); t += 32) {
+                const int k = S.flag[t];
+                const int c = clip_exact_row(S, p, N, box, a.box_lo, k, m, delta, &close);
+                amb |= c == 2;
+                if (c == 1) {
+                    const int q = atomicAdd(&S.nviol, 1);
+                    if (q < 32) S.viol[q] = k;
+                    else amb = true;
+                }
+            }
+            if (__any_sync(FULL, amb)) { fallback = true; break; }
+            __syncwarp();
+            const int nv = S.nviol;
+            if (nv == 0) break;
+            if (++rounds >= kWMaxFix) { fallback = true; break; }
+            // another round: the edges and the violated rows
+            kk[0] = lane < m ? id : -1;
+            kk[1] = lane < nv ? S.viol[lane] : -1;
+            kk[2] = -1;
+            __syncwarp();
         }
-        // an FP32 pass that emptied the polygon proves nothing: the FP64 fallback decides
-        if (m == 0) fallback = true;
-        if (!fallback) fallback = !wfinal(S, m, buf, rv);
+        n_cuts += ncut;
         if (!fallback && a.chk && m <= kChkMaxV) {
             // the dense check runs on the tensor cores (check_tc); the finish pass emits the cell
-            unsigned long long p = 0;
-            if (lane == 0) p = atomicAdd(a.chk_count, 1ull);
-            p = __shfl_sync(FULL, p, 0);
-            CheckRec &R = a.chk[p];
+            unsigned long long q = 0;
+            if (lane == 0) q = atomicAdd(a.chk_count, 1ull);
+            q = __shfl_sync(FULL, q, 0);
+            CheckRec &R = a.chk[q];
             if (lane == 0) { R.cell = (int32_t)cell; R.m = m; }
-            for (int i = lane; i < m; i += 32) {
-                R.pe[i] = S.pe[buf][i];
-                R.v[i][0] = S.pv[buf][i][0]; R.v[i][1] = S.pv[buf][i][1]; R.v[i][2] = S.pv[buf][i][2];
+            if (lane < m) {
+                R.pe[lane] = S.pe[lane];
+                R.v[lane][0] = S.pv[lane][0]; R.v[lane][1] = S.pv[lane][1]; R.v[lane][2] = S.pv[lane][2];
             }
-            n_cuts += (unsigned long long)ncut;
-            __syncwarp();
             continue;
         }
-        // ---- the all-row check, certified; violators are cut in (FP64) and the check repeats
-        int rounds = 0, cell_close = 0;
-        if (!fallback) fallback = wcheck(a, S, rv, N, m, buf, rounds, ncut, cell_close);
         if (fallback) {
             // the block kernel solves this cell (double-float, then FP64 where needed)
             if (lane == 0) {
-                const unsigned long long p = atomicAdd(a.fb_count, 1ull);
-                a.fb_list[p] = (int32_t)cell;
+                const unsigned long long q = atomicAdd(a.fb_count, 1ull);
+                a.fb_list[q] = (int32_t)cell;
             }
             n_fb += 1;
             continue;
         }
-        // ---- a6 emit, a7 march
-        const bool emitted = wemit(a, S, cell, net_id, N, m, buf);
+        // ---- a6 emit: the face's area in FP32 where that is clear of every rounding, else in FP64
+        const float nxv = __shfl_sync(FULL, vx, lane + 1 < m ? lane + 1 : 0), nyv = __shfl_sync(FULL, vy, lane + 1 < m ? lane + 1 : 0);
+        float area = lane < m ? vx * nyv - nxv * vy - 1e-5f * (fabsf(vx * nyv) + fabsf(nxv * vy)) : 0.0f;
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) area += __shfl_xor_sync(FULL, area, o);
+        int emit = area > 1e-11f || clip_area(S, m, a.box) ? m : 0;
+        if (emit > ar.maxv) {
+            if (lane == 0) atomicOr(ar.counters + kStatus, kStFaceVerts);
+            emit = 0;
+        }
+        if (lane == 0) ar.nverts[cell] = emit;
         n_solved += 1;
-        if (!emitted) n_empty += 1;
+        if (!emit) n_empty += 1;
         if (rounds) n_fix += 1;
-        n_cuts += (unsigned long long)ncut;
-        n_close += (unsigned long long)cell_close;
-        __syncwarp();
+        n_close += (unsigned)close;                      // per lane, summed at the end
+        if (!emit) continue;
+#pragma unroll 1
+        for (int i = lane; i < 3 * m; i += 32) ar.verts[cell * ar.maxv * 3 + i] = (&S.pv[0][0])[i];
+        const int e = lane < m ? S.pe[lane] : N;
+        if (lane < m) ar.edges[cell * ar.maxv + lane] = e;
+        // ---- a7 march: each neuron edge pushes its neighbour, entered at the shared edge's midpoint
+        const float4 v0 = S.vf[lane < m ? lane : 0], v1 = S.vf[lane + 1 < m ? lane + 1 : 0];
+        insert_neighbors_level(ar, S.key, cell, net_id, e < N, (unsigned)e, __ldcg(ar.hash + cell) ^ (e < N ? __ldg(ar.zob + e) : 0ull),
+                               0.5f * (v0.x + v1.x), 0.5f * (v0.y + v1.y), 0.5f * (v0.z + v1.z));
     }
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) n_close += __shfl_xor_sync(FULL, n_close, o);
     if (lane == 0) {
         unsigned long long *C = ar.counters;
-        if (n_solved) atomicAdd(C + kSolved, n_solved);
-        if (n_empty) atomicAdd(C + kEmpty, n_empty);
-        if (n_fix) atomicAdd(C + kFixups, n_fix);
-        if (n_cuts) atomicAdd(C + kCuts, n_cuts);
-        if (n_close) atomicAdd(C + kCloseCalls, n_close);
-        if (n_fb) atomicAdd(C + kWarpFallback, n_fb);
+        if (n_solved) atomicAdd(C + kSolved, (unsigned long long)n_solved);
+        if (n_empty) atomicAdd(C + kEmpty, (unsigned long long)n_empty);
+        if (n_fix) atomicAdd(C + kFixups, (unsigned long long)n_fix);
+        if (n_cuts) atomicAdd(C + kCuts, (unsigned long long)n_cuts);
+        if (n_close) atomicAdd(C + kCloseCalls, (unsigned long long)n_close);
+        if (n_fb) atomicAdd(C + kWarpFallback, (unsigned long long)n_fb);
     }
 }
 
@@ -658,18 +972,20 @@ __global__ void __launch_bounds__(kWW * 32) clip_warp_finish_kernel(MarchArgs a)
     }
 }
 
+static int clip_smem_bytes() { return kWW * (int)sizeof(ClipSh); }
+
 static int g_clip_resident = 0;       // clip_warp_kernel blocks resident on the whole GPU at once
 
 cudaError_t prepare_clip_warp()
 {
-    cudaError_t e = cudaFuncSetAttribute(clip_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, warp_smem_bytes());
+    cudaError_t e = cudaFuncSetAttribute(clip_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, clip_smem_bytes());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(clip_warp_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, warp_smem_bytes());
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, clip_warp_kernel, kWW * 32, warp_smem_bytes());
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, clip_warp_kernel, kWW * 32, clip_smem_bytes());
     if (e != cudaSuccess) return e;
     g_clip_resident = std::max(1, sms * per_sm);
     return cudaSuccess;
@@ -681,7 +997,7 @@ void launch_clip_warp(const MarchArgs &a, cudaStream_t st)
     // with a work counter: one resident wave that drains the cells; else one warp per cell
     const int64_t cap = a.work && g_clip_resident > 0 ? g_clip_resident : 152 * 64;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + kWW - 1) / kWW, cap));
-    clip_warp_kernel<<<grid, kWW * 32, warp_smem_bytes(), st>>>(a);
+    clip_warp_kernel<<<grid, kWW * 32, clip_smem_bytes(), st>>>(a);
 }
 
 void launch_clip_warp_finish(const MarchArgs &a, cudaStream_t st)
