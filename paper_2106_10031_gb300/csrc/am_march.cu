@@ -673,6 +673,10 @@ __device__ __forceinline__ int df_split(int nl)
     return nl <= 8 ? 3 : nl <= 16 ? 2 : nl <= kNarrow ? 1 : nl <= kT / 4 ? 2 : nl <= kT / 2 ? 1 : 0;
 }
 
+// The partial sums of a row that its error bound allows for: a block's threads shared out, whatever
+// df_split (never more) takes, so that a bound depends on the net alone.
+__device__ __forceinline__ int df_parts(int nl) { return nl >= kT ? 1 : kT / nl; }
+
 // Rows of every layer.  FP64: one thread per row and column (k, c), the four columns of a row in
 // neighbouring lanes, so a layer of n rows issues 4 n / 32 chains of its active units and nothing
 // else on the FP64 pipe, whose warp instructions take about 64 cycles each whatever the lanes do
@@ -703,7 +707,7 @@ __device__ __forceinline__ void compose(const NetDev &netg, const Sh &s, bool tc
             int nact = 0;
 #pragma unroll 1
             for (int w = 0; w < n1; w += 32) nact += __popc(s.mask[w >> 5] & (n1 - w < 32 ? (1u << (n1 - w)) - 1u : ~0u));
-            const float g = df_gamma(nact + (net.L > 1 ? 1 << df_split(net.width[2]) : 1) + 2);
+            const float g = df_gamma(nact + (net.L > 1 ? df_parts(net.width[2]) : 1) + 2);
 #pragma unroll 1
             for (int i0 = 0; i0 < 4 * n1; i0 += kT) {
                 const int i = i0 + tid, k = i >> 2;
@@ -775,8 +779,8 @@ __device__ __forceinline__ void compose(const NetDev &netg, const Sh &s, bool tc
         } else {
             const float *Ah = net.h + net.offA[l], *Al = net.l + net.offA[l];
             const int sh = df_split(nl), S = 1 << sh;
-            const float g = df_gamma(t1 - t0 + S + 2);
-            const float gn = l < net.L ? df_gamma(s.lst0[l + 1] - t1 + (1 << df_split(net.width[l + 1])) + 2) : 0.0f;
+            const float g = df_gamma(t1 - t0 + df_parts(nl) + 2);
+            const float gn = l < net.L ? df_gamma(s.lst0[l + 1] - t1 + df_parts(net.width[l + 1]) + 2) : 0.0f;
             if (nl <= kNarrow) {
                 // one lane per row, column and part of the sum, in one pass of the block
                 const int sp = tid & (S - 1), c = (tid >> sh) & 3, k = tid >> (sh + 2);

@@ -185,3 +185,30 @@ def test_sliced_compose_edge_cases(oracle_mod):
         assert e.value.status == 1
         with pytest.raises(am.AMError):
             m.set_tuning(compose_tile_cells=24)
+
+
+@pytest.mark.parametrize("widths", [(8, 16, 33, 9), (12, 70, 17, 128), (130, 100, 256, 31)])
+def test_double_float_bounds_follow_their_recursion(oracle_mod, widths):
+    """The bound of a row as it is defined, whatever lanes share the row's sum:
+        e_1 = 2 u^2 |C_1|_1,  e_l,k = sum_j |W_kj| (e_j + g |z_j|_1) + g |C_k|_1,  each times 1.01 or so,
+    over the active j, g = 2 (n_active + max(1, 256 // n_l) + 6)^2 u^2, u = 2^-24.  The kernel's sums
+    round up: at most 256 units of 2^-23 per layer, over four layers 1.3e-4."""
+    import paper_2106_10031_gb300 as am
+    mlp = tiny_net(widths, 7)
+    rng = np.random.default_rng(4)
+    S = rng.integers(0, 2, (3, mlp.N)).astype(np.uint8)
+    with am.Mesher(max_cells=1 << 10, max_neurons=1024, max_width=256) as m:
+        rows, err = m.compose(m.load_mlp(mlp), _keys_from_states(S, mlp.N), "mixed")
+    u2, row0 = 2.0 ** -48, np.concatenate([[0], np.cumsum(mlp.widths)])
+    for s, r, got in zip(S, rows, err):
+        l1 = np.abs(r).sum(axis=1)
+        want = np.zeros(mlp.N)
+        c1 = np.abs(mlp.weights[0][:, :3]).sum(1) + np.abs(mlp.biases[0])
+        want[:widths[0]] = 2 * u2 * c1 * 1.01
+        for l in range(1, mlp.L):
+            p, q = slice(row0[l - 1], row0[l]), slice(row0[l], row0[l + 1])
+            on = s[p] == 1
+            g = 2 * (on.sum() + max(1, 256 // widths[l]) + 6.0) ** 2 * u2
+            carry = (want[p] + g * l1[p] * 1.001)[on]
+            want[q] = (np.abs(mlp.weights[l])[:, on] @ carry + g * np.abs(mlp.biases[l])) * 1.01
+        np.testing.assert_allclose(got[:mlp.N], want, rtol=1.3e-4)
