@@ -197,8 +197,8 @@ struct ProposalDev {
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;   // FP32 master weights, grads, Adam state
     __nv_bfloat16 *wb = nullptr, *w2t = nullptr, *w3t = nullptr;     // BF16 copies
     float *buf[8] = {};
-    __nv_bfloat16 *bbuf[4] = {};
-    float *loss_parts = nullptr;
+    __nv_bfloat16 *bbuf[6] = {};
+    float *loss_parts = nullptr, *losses = nullptr;
     PropTC tc;                     // forward pass on the tensor cores (when the shape allows)
 };
 cudaError_t proposal_alloc(ProposalDev &p, int n_in, int hidden, int n_out, int max_batch);

@@ -7,8 +7,7 @@
 //   training loss: mean binary cross-entropy of sigmoid(z) against the 0/1 boundary labels.
 //
 // Training is mixed precision: FP32 master weights, BF16 operands for every matrix product,
-// FP32 accumulation, Adam.  Matrix products use one tiled kernel (64 x 64 output tile per
-// block, 16-deep K slices staged in shared memory).
+// FP32 accumulation, Adam.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -19,62 +18,308 @@
 
 namespace am {
 
-constexpr int kGT = 64;     // GEMM output tile
-constexpr int kGK = 16;     // GEMM K slice
+// ---- products of BF16 operands on the FP32 pipes
+//
+// Every element is one chain of fused multiply-adds over k in ascending order from zero, so a result does
+// not depend on the tile, the launch or the device's load (a split of k, or the tensor cores' own order,
+// would move the BF16 roundings between the layers).  What bounds a training step of this MLP (batch 1024,
+// 15 -> 256 -> 256 -> 2048: 1.8 G multiply-adds, 46 us at the FP32 peak) is keeping the FP32 pipes fed
+// along chains of up to 2048 k: slices of 32 k are staged in shared memory as FP32, the next two slices'
+// loads in flight while one is multiplied, the operands of the next k read while those of one are
+// multiplied, each thread keeps a TM x TN block of sums, and the products that wait for the same input
+// share one launch, with their bias, activation, loss or backward step as the epilogue.  A step takes
+// 291 us; 933 with a 64 x 64 kernel per product (4 loads per 8 multiply-adds, strided global reads), its
+// element-wise kernels and a copy of the loss to the host per step.
 
-// C[M x N] = alpha * op(A)[M x K] * op(B)[K x N] + beta * C.  A is row-major M x K (lda = K) or,
-// with ta, stored K x M (lda = M); B is row-major K x N (ldb = N) or, with tb, stored N x K.
-__global__ void __launch_bounds__(256) gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16 *A, int lda,
-                                                        bool ta, const __nv_bfloat16 *B, int ldb, bool tb, float *C,
-                                                        int ldc, float alpha, float beta)
+constexpr int kGK = 32;     // K slice
+constexpr int kLossSteps = 4096;     // losses kept on the device between copies
+
+enum { kEpiStore = 0, kEpiBias = 1, kEpiBiasRelu = 2, kEpiBce = 3, kEpiReluBack = 4, kEpiColsum = 5 };
+
+// C[M x N] = op(A)[M x K] op(B)[K x N] and an epilogue.  A is row-major M x K (lda = K) or, with ta, stored
+// K x M (lda = M); B is row-major K x N (ldb = N) or, with tb, stored N x K.
+struct GemmJob {
+    int M, N, K, lda, ldb, ta, tb, epi;
+    int ldc, ldy;                 // row strides of C and H, and of Y
+    int va, vb;                   // A, B: rows of 16-byte pieces (8 | ld, 16-byte aligned)
+    const __nv_bfloat16 *A, *B;
+    float *C;
+    const float *bias;            // kEpiBias, kEpiBiasRelu, kEpiBce: per column
+    __nv_bfloat16 *H;             // BF16 result: activations (kEpiBiasRelu), dz (kEpiBce), da (kEpiReluBack)
+    const float *Y;               // kEpiBce: labels, kEpiReluBack: the layer's pre-activations
+    float scale;                  // kEpiBce: 1 / (rows cols)
+    float *loss_parts;            // kEpiBce: one sum of softplus(z) - y z per tile
+};
+constexpr int kMaxJobs = 3;
+struct GemmJobs {
+    GemmJob j[kMaxJobs];
+    int first[kMaxJobs + 1];      // first tile of each job (kEpiColsum: blocks of 32 columns)
+    int n;
+};
+
+// db[c] = sum over rows of C[r, c]: 32 columns per block, the rows in groups combined in shared memory
+template <int T>
+__device__ __forceinline__ void colsum_block(const GemmJob &g, int tile, float *sh)
 {
-    __shared__ float As[kGK][kGT + 1];
-    __shared__ float Bs[kGK][kGT + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int row0 = blockIdx.y * kGT, col0 = blockIdx.x * kGT;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += kGK) {
-        for (int i = threadIdx.x; i < kGK * kGT; i += 256) {
-            const int kk = i / kGT, mm = i % kGT;
-            const int gr = row0 + mm, gk = k0 + kk;
-            float va = 0.0f, vb = 0.0f;
-            if (gr < M && gk < K) va = __bfloat162float(ta ? A[(size_t)gk * lda + gr] : A[(size_t)gr * lda + gk]);
-            const int gc = col0 + mm;
-            if (gc < N && gk < K) vb = __bfloat162float(tb ? B[(size_t)gc * ldb + gk] : B[(size_t)gk * ldb + gc]);
-            As[kk][mm] = va;
-            Bs[kk][mm] = vb;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < kGK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty + 16 * i]; b[i] = Bs[kk][tx + 16 * i]; }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
+    constexpr int G = T / 32;
+    const int c = tile * 32 + (threadIdx.x & 31), q = threadIdx.x >> 5;
+    float s = 0.0f;
+    if (c < g.N) {
+#pragma unroll 8
+        for (int r = q; r < g.M; r += G) s += g.C[(size_t)r * g.ldc + c];
     }
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    if (q == 0 && c < g.N) {
+        for (int w = 1; w < G; ++w) s += sh[threadIdx.x + 32 * w];
+        const_cast<float *>(g.bias)[c] = s;          // the job's output vector
+    }
+}
+
+// 8 consecutive BF16 elements at p (n of them inside the matrix, none if n <= 0).  The 16-byte form is one
+// predicated load and nothing looks at its value: the elements past n, which the row's stride covers, are
+// zeroed by tail8 when the slice is stored.  (With the mask here every load was waited for where it was
+// issued, and a slice of 32 k took two trips to L2 longer: 332 us per step of 1024 samples.)
+__device__ __forceinline__ void load8(uint4 &v, const __nv_bfloat16 *p, int n, bool vec)
+{
+    v = make_uint4(0u, 0u, 0u, 0u);
+    if (vec) {
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.gt.s32 q, %5, 0;\n\t@q ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                     : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"(n) : "memory");
+        return;
+    }
+    unsigned w[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < 4; ++j) {
+        const unsigned lo = 2 * j < n ? __bfloat16_as_ushort(p[2 * j]) : 0u;
+        const unsigned hi = 2 * j + 1 < n ? __bfloat16_as_ushort(p[2 * j + 1]) : 0u;
+        w[j] = lo | (hi << 16);
+    }
+    v = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__device__ __forceinline__ uint4 tail8(uint4 v, int n)
+{
+    if (n < 8) {
+        unsigned *w = &v.x;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-            if (r < M && c < N) {
-                float *p = C + (size_t)r * ldc + c;
-                *p = alpha * acc[i][j] + (beta != 0.0f ? beta * *p : 0.0f);
-            }
+            if (2 * j >= n) w[j] = 0u;
+            else if (2 * j + 1 >= n) w[j] &= 0xffffu;
         }
+    }
+    return v;
 }
 
-static void gemm(int M, int N, int K, const __nv_bfloat16 *A, int lda, bool ta, const __nv_bfloat16 *B, int ldb,
-                 bool tb, float *C, int ldc, float alpha, float beta, cudaStream_t st)
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_jobs_kernel(const __grid_constant__ GemmJobs jobs)
 {
-    dim3 grid((N + kGT - 1) / kGT, (M + kGT - 1) / kGT);
-    gemm_bf16_kernel<<<grid, 256, 0, st>>>(M, N, K, A, lda, ta, B, ldb, tb, C, ldc, alpha, beta);
+    constexpr int T = (BM / TM) * (BN / TN), CX = BN / TN;
+    constexpr int LA = BM + 4, LB = BN + 4;          // row strides: 16-byte rows
+    static_assert(BM == BN && BM * kGK / 8 == T && BM % 32 == 0, "one 16-byte piece of A and of B per thread and slice");
+    __shared__ __align__(16) float As[2][kGK][LA];
+    __shared__ __align__(16) float Bs[2][kGK][LB];
+    int ji = 0;
+    while (ji + 1 < jobs.n && (int)blockIdx.x >= jobs.first[ji + 1]) ++ji;
+    const GemmJob &g = jobs.j[ji];
+    const int tile = (int)blockIdx.x - jobs.first[ji];
+    if (g.epi == kEpiColsum) {
+        colsum_block<T>(g, tile, &As[0][0][0]);
+        return;
+    }
+    const int tiles_n = (g.N + BN - 1) / BN;
+    const int row0 = tile / tiles_n * BM, col0 = tile % tiles_n * BN;
+    const int tid = threadIdx.x, tx = tid % CX, ty = tid / CX, lane = tid & 31, warp = tid >> 5;
+    // a thread's piece of a slice.  Stored k-contiguous: 8 k of row km, the rows along the lanes (the
+    // stores of one k then fall in 32 banks); stored m-contiguous: 8 rows from mm of k = mk
+    const int km = tid % BM, kq = 8 * (tid / BM), mm = 8 * (tid % (BM / 8)), mk = tid / (BM / 8);
+    const int M = g.M, N = g.N, K = g.K;
+    // elements of a thread's piece inside the matrix, and its place
+    auto inside = [&](bool mfirst, int m0, int m_end, int k0) {
+        if (mfirst) return k0 + mk < K ? m_end - (m0 + mm) : 0;
+        return m0 + km < m_end ? K - (k0 + kq) : 0;
+    };
+    auto place = [&](const __nv_bfloat16 *X, int ld, bool mfirst, int m0, int k0) {
+        return mfirst ? X + (size_t)(k0 + mk) * ld + m0 + mm : X + (size_t)(m0 + km) * ld + k0 + kq;
+    };
+    auto put = [&](float *S, int ls, bool mfirst, const uint4 v) {
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            f[2 * j] = __uint_as_float(w[j] << 16);
+            f[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
+        }
+        if (mfirst) {
+            float4 *o = reinterpret_cast<float4 *>(S + mk * ls + mm);
+            o[0] = make_float4(f[0], f[1], f[2], f[3]);
+            o[1] = make_float4(f[4], f[5], f[6], f[7]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) S[(kq + j) * ls + km] = f[j];
+        }
+    };
+    uint4 ra[2], rb[2];              // the slices of k0 + 32 and k0 + 64
+    auto load = [&](uint4 &a, uint4 &b, int k0) {
+        if (k0 >= K) return;
+        load8(a, place(g.A, g.lda, g.ta, row0, k0), inside(g.ta, row0, M, k0), g.va);
+        load8(b, place(g.B, g.ldb, !g.tb, col0, k0), inside(!g.tb, col0, N, k0), g.vb);
+    };
+    auto store = [&](int buf, const uint4 &a, const uint4 &b, int k0) {
+        if (k0 >= K) return;
+        put(&As[buf][0][0], LA, g.ta, tail8(a, inside(g.ta, row0, M, k0)));
+        put(&Bs[buf][0][0], LB, !g.tb, tail8(b, inside(!g.tb, col0, N, k0)));
+    };
+    float acc[TM][TN] = {};
+    auto multiply = [&](const int buf) {
+        // operands of k + D in flight while those of k are multiplied: shared memory answers after 34
+        // cycles, and few warps share a scheduler
+        constexpr int D = TM == 4 ? 2 : 4;
+        float av[D][TM], bv[D][TN];
+        auto operands = [&](int kk) {
+            if constexpr (TM == 4) *reinterpret_cast<float4 *>(av[kk % D]) = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * TM]);
+            else *reinterpret_cast<float2 *>(av[kk % D]) = *reinterpret_cast<const float2 *>(&As[buf][kk][ty * TM]);
+            *reinterpret_cast<float4 *>(bv[kk % D]) = *reinterpret_cast<const float4 *>(&Bs[buf][kk][tx * TN]);
+        };
+#pragma unroll
+        for (int kk = 0; kk < D; ++kk) operands(kk);
+#pragma unroll
+        for (int kk = 0; kk < kGK; ++kk) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(av[kk % D][i], bv[kk % D][j], acc[i][j]);
+            if (kk + D < kGK) operands(kk + D);
+        }
+    };
+    load(ra[0], rb[0], 0);
+    load(ra[1], rb[1], kGK);
+    store(0, ra[0], rb[0], 0);
+    __syncthreads();
+    for (int k0 = 0; k0 < K; k0 += 2 * kGK) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = k0 + h * kGK;
+            if (k >= K) break;
+            load(ra[h], rb[h], k + 2 * kGK);
+            multiply(h);
+            store(h ^ 1, ra[h ^ 1], rb[h ^ 1], k + kGK);
+            __syncthreads();
+        }
+    }
+    float part = 0.0f;
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int r = row0 + ty * TM + i, c = col0 + tx * TN + j;
+            if (r >= g.M || c >= g.N) continue;
+            const size_t o = (size_t)r * g.ldc + c;
+            const float v = acc[i][j] + 0.0f;
+            if (g.epi == kEpiStore) {
+                g.C[o] = v;
+            } else if (g.epi == kEpiBias) {
+                g.C[o] = v + g.bias[c];
+            } else if (g.epi == kEpiBiasRelu) {
+                const float z = v + g.bias[c];
+                g.C[o] = z;
+                g.H[o] = __float2bfloat16_rn(fmaxf(z, 0.0f));
+            } else if (g.epi == kEpiBce) {
+                // dz = (sigmoid(z) - y) / (rows cols), and this element of the loss
+                const float z = v + g.bias[c], y = g.Y[(size_t)r * g.ldy + c];
+                part += (z > 0.0f ? z + log1pf(expf(-z)) : log1pf(expf(z))) - y * z;
+                const float d = (1.0f / (1.0f + expf(-z)) - y) * g.scale;
+                g.H[o] = __float2bfloat16_rn(d);
+                g.C[o] = d;
+            } else {
+                // da = dh (a > 0)
+                const float d = g.Y[(size_t)r * g.ldy + c] > 0.0f ? v : 0.0f;
+                g.H[o] = __float2bfloat16_rn(d);
+                g.C[o] = d;
+            }
+        }
+    if (g.epi == kEpiBce) {
+        float *red = &As[0][0][0];
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0) red[warp] = part;
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < T / 32; ++w) part += red[w];
+            g.loss_parts[tile] = part;
+        }
+    }
 }
+
+// the products of one launch
+struct JobList {
+    GemmJobs q{};
+    void add(const GemmJob &g) { q.j[q.n++] = g; }
+    void run(cudaStream_t st)
+    {
+        // 64 x 64 tiles (3 shared-memory wavefronts per 16 multiply-adds of a warp) when they fill the
+        // chip twice, else 32 x 32 (four times as many, of half the threads): the logits of 1024 samples
+        // take 50 us in 512 large tiles, dW3 and dh2 124 us in 832 small ones where 192 large ones leave
+        // most schedulers one warp.  One 64 x 32 tile for both took 3.12 ms for 8 steps against 2.66.
+        auto tiles = [&](int B) {
+            int t = 0;
+            for (int i = 0; i < q.n; ++i) {
+                const GemmJob &g = q.j[i];
+                q.first[i] = t;
+                t += g.epi == kEpiColsum ? (g.N + 31) / 32 : ((g.M + B - 1) / B) * ((g.N + B - 1) / B);
+            }
+            q.first[q.n] = t;
+            return t;
+        };
+        int t = tiles(64);
+        if (t >= 2 * 152) {
+            gemm_jobs_kernel<64, 64, 4, 4><<<t, 256, 0, st>>>(q);
+        } else {
+            t = tiles(32);
+            gemm_jobs_kernel<32, 32, 2, 4><<<t, 128, 0, st>>>(q);
+        }
+        q = GemmJobs{};
+    }
+};
+
+static GemmJob product(int M, int N, int K, const __nv_bfloat16 *A, int lda, bool ta, const __nv_bfloat16 *B, int ldb,
+                       bool tb, float *C, int epi)
+{
+    GemmJob g{};
+    g.M = M; g.N = N; g.K = K;
+    g.A = A; g.lda = lda; g.ta = ta;
+    g.B = B; g.ldb = ldb; g.tb = tb;
+    g.C = C;
+    g.ldc = g.ldy = N;
+    g.epi = epi;
+    g.va = lda % 8 == 0 && (uintptr_t)A % 16 == 0;
+    g.vb = ldb % 8 == 0 && (uintptr_t)B % 16 == 0;
+    return g;
+}
+
+static GemmJob column_sum(const float *G, int rows, int cols, int ld, float *db)
+{
+    GemmJob g{};
+    g.M = rows; g.N = cols;
+    g.ldc = ld;
+    g.C = const_cast<float *>(G);
+    g.bias = db;
+    g.epi = kEpiColsum;
+    return g;
+}
+
+static int blocks_for(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
+
+// BF16 copy of a rows x cols matrix with row stride ld >= cols (the padding is zero)
+__global__ void pad_bf16_kernel(const float *x, int rows, int cols, int ld, __nv_bfloat16 *y)
+{
+    const int64_t n = (int64_t)rows * ld;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i % ld);
+        y[i] = __float2bfloat16_rn(c < cols ? x[i / ld * cols + c] : 0.0f);
+    }
+}
+
+static int up8(int n) { return (n + 7) & ~7; }      // row stride of the activations: 16-byte pieces
 
 __global__ void to_bf16_kernel(const float *x, __nv_bfloat16 *y, int64_t n)
 {
@@ -82,58 +327,19 @@ __global__ void to_bf16_kernel(const float *x, __nv_bfloat16 *y, int64_t n)
         y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// Z (rows x cols) += bias; H = relu(Z) in BF16 (pre-activations kept for the backward pass)
-__global__ void bias_relu_kernel(float *Z, const float *b, __nv_bfloat16 *H, int rows, int cols, int relu)
+// losses[it] = the sum of n partial sums (FP64) over count, for a training step; one block
+__global__ void loss_kernel(const float *parts, int n, double count, float *loss)
 {
-    const int64_t n = (int64_t)rows * cols;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float z = Z[i] + b[i % cols];
-        Z[i] = z;
-        if (H) H[i] = __float2bfloat16_rn(relu ? fmaxf(z, 0.0f) : z);
-    }
-}
-
-// dZ = (sigmoid(z) - y) / (rows cols) in BF16; per-block partial sums of softplus(z) - y z
-__global__ void bce_kernel(const float *Z, const float *Y, __nv_bfloat16 *dZ, float *dZf, int64_t n, float scale,
-                           float *loss_parts)
-{
-    __shared__ float red[256];
-    float acc = 0.0f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float z = Z[i], y = Y[i];
-        const float sp = z > 0.0f ? z + log1pf(expf(-z)) : log1pf(expf(z));
-        acc += sp - y * z;
-        const float g = (1.0f / (1.0f + expf(-z)) - y) * scale;
-        dZ[i] = __float2bfloat16_rn(g);
-        if (dZf) dZf[i] = g;
-    }
-    red[threadIdx.x] = acc;
+    __shared__ double red[8];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) s += (double)parts[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)blockDim.x / 32; ++w) s += red[w];
+        *loss = (float)(s / count);
     }
-    if (threadIdx.x == 0) loss_parts[blockIdx.x] = red[0];
-}
-
-// dA = dH * (A > 0) (FP32 in, BF16 and FP32 out)
-__global__ void relu_back_kernel(const float *dH, const float *A, __nv_bfloat16 *dA, float *dAf, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float g = A[i] > 0.0f ? dH[i] : 0.0f;
-        dA[i] = __float2bfloat16_rn(g);
-        dAf[i] = g;
-    }
-}
-
-// db[c] = sum over rows of G[r, c]
-__global__ void colsum_kernel(const float *G, int rows, int cols, float *db)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.0f;
-    for (int r = 0; r < rows; ++r) s += G[(size_t)r * cols + c];
-    db[c] = s;
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master weights, then the BF16 copy
@@ -222,7 +428,6 @@ void launch_proposal_samples(const SampleArgs &a, cudaStream_t st)
     if (blocks > 0) proposal_samples_kernel<<<(int)blocks, 256, 0, st>>>(a);
 }
 
-static int blocks_for(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
 
 // ------------------------------------------------------------------------------------------
 
@@ -246,12 +451,14 @@ cudaError_t proposal_alloc(ProposalDev &p, int n_in, int hidden, int n_out, int 
     if ((e = cudaMalloc(&p.wb, sizeof(__nv_bfloat16) * tot))) return e;
     if ((e = cudaMalloc(&p.w2t, sizeof(__nv_bfloat16) * hidden * hidden))) return e;
     if ((e = cudaMalloc(&p.w3t, sizeof(__nv_bfloat16) * hidden * (n_out + 1)))) return e;
-    const int64_t act = (int64_t)max_batch * std::max(std::max(hidden, n_out), n_in);
+    const int64_t act = (int64_t)max_batch * up8(std::max(std::max(hidden, n_out), n_in));
     for (int i = 0; i < 8; ++i)
         if ((e = cudaMalloc(&p.buf[i], sizeof(float) * act))) return e;
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 6; ++i)
         if ((e = cudaMalloc(&p.bbuf[i], sizeof(__nv_bfloat16) * act))) return e;
-    if ((e = cudaMalloc(&p.loss_parts, sizeof(float) * 152 * 16))) return e;
+    const int64_t tiles = (int64_t)((max_batch + 31) / 32) * ((n_out + 31) / 32);
+    if ((e = cudaMalloc(&p.loss_parts, sizeof(float) * tiles))) return e;
+    if ((e = cudaMalloc(&p.losses, sizeof(float) * kLossSteps))) return e;
     // the forward pass of whole batches on the tensor cores (inference: am_proposal_forward and
     // the level march), when the shape allows it; W2 and W3 are read in place from the BF16 copy
     return prop_tc_alloc(p.tc, n_in, hidden, n_out, std::max(max_batch, 4096), p.wb + p.off[2], p.wb + p.off[4]);
@@ -259,12 +466,12 @@ cudaError_t proposal_alloc(ProposalDev &p, int n_in, int hidden, int n_out, int 
 
 void proposal_free(ProposalDev &p)
 {
-    void *b[] = {p.w, p.g, p.m, p.v, p.wb, p.w2t, p.w3t, p.loss_parts};
+    void *b[] = {p.w, p.g, p.m, p.v, p.wb, p.w2t, p.w3t, p.loss_parts, p.losses};
     for (void *x : b)
         if (x) cudaFree(x);
     for (int i = 0; i < 8; ++i)
         if (p.buf[i]) cudaFree(p.buf[i]);
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 6; ++i)
         if (p.bbuf[i]) cudaFree(p.bbuf[i]);
     prop_tc_free(p.tc);
     p = ProposalDev{};
@@ -281,40 +488,65 @@ void proposal_sync_copies(ProposalDev &p, cudaStream_t st)
     prop_tc_sync_weights(p.tc, p.w + p.off[0], st);
 }
 
-// Forward pass over B samples (B <= max_batch).  Activations: buf0 a1, buf1 a2, buf2 z (FP32);
-// bbuf0 x, bbuf1 h1, bbuf2 h2 (BF16).
-static void forward(ProposalDev &p, const float *X, int B, cudaStream_t st)
+// Forward pass over B samples (B <= max_batch).  Activations: buf0 a1, buf1 a2 (FP32, for the backward
+// pass); bbuf0 x, bbuf1 h1, bbuf2 h2 (BF16).  Without labels the logits go to buf2; with labels Y the loss's
+// partial sums to loss_parts and dz to buf3 (FP32) and bbuf3 (BF16).
+static void forward(ProposalDev &p, const float *X, const float *Y, int B, cudaStream_t st)
 {
     const int H = p.hidden, I = p.n_in, O = p.n_out;
     const __nv_bfloat16 *W1 = p.wb + p.off[0], *W2 = p.wb + p.off[2], *W3 = p.wb + p.off[4];
-    to_bf16_kernel<<<blocks_for((int64_t)B * I), 256, 0, st>>>(X, p.bbuf[0], (int64_t)B * I);
-    gemm(B, H, I, p.bbuf[0], I, false, W1, I, true, p.buf[0], H, 1.0f, 0.0f, st);          // a1 = X W1^T
-    bias_relu_kernel<<<blocks_for((int64_t)B * H), 256, 0, st>>>(p.buf[0], p.w + p.off[1], p.bbuf[1], B, H, 1);
-    gemm(B, H, H, p.bbuf[1], H, false, W2, H, true, p.buf[1], H, 1.0f, 0.0f, st);          // a2 = h1 W2^T
-    bias_relu_kernel<<<blocks_for((int64_t)B * H), 256, 0, st>>>(p.buf[1], p.w + p.off[3], p.bbuf[2], B, H, 1);
-    gemm(B, O, H, p.bbuf[2], H, false, W3, H, true, p.buf[2], O, 1.0f, 0.0f, st);          // z = h2 W3^T
-    bias_relu_kernel<<<blocks_for((int64_t)B * O), 256, 0, st>>>(p.buf[2], p.w + p.off[5], nullptr, B, O, 0);
+    JobList q;
+    pad_bf16_kernel<<<blocks_for((int64_t)B * up8(I)), 256, 0, st>>>(X, B, I, up8(I), p.bbuf[0]);
+    GemmJob g = product(B, H, I, p.bbuf[0], up8(I), false, W1, I, true, p.buf[0], kEpiBiasRelu);          // a1 = X W1^T + b1
+    g.bias = p.w + p.off[1];
+    g.H = p.bbuf[1];
+    q.add(g);
+    q.run(st);
+    g = product(B, H, H, p.bbuf[1], H, false, W2, H, true, p.buf[1], kEpiBiasRelu);                  // a2 = h1 W2^T + b2
+    g.bias = p.w + p.off[3];
+    g.H = p.bbuf[2];
+    q.add(g);
+    q.run(st);
+    g = product(B, O, H, p.bbuf[2], H, false, W3, H, true, Y ? p.buf[3] : p.buf[2], Y ? kEpiBce : kEpiBias);   // z = h2 W3^T + b3
+    g.bias = p.w + p.off[5];
+    g.H = p.bbuf[3];
+    g.Y = Y;
+    if (Y) g.ldc = up8(O);
+    g.scale = 1.0f / (float)((int64_t)B * O);
+    g.loss_parts = p.loss_parts;
+    q.add(g);
+    q.run(st);
 }
 
-// Loss and gradients (into p.g) over B samples; returns the number of loss partial blocks.
-static int backward(ProposalDev &p, const float *Y, int B, cudaStream_t st)
+// partial sums of the loss that a forward pass over B samples leaves (as JobList::run tiles it)
+static int loss_tiles(const ProposalDev &p, int B)
+{
+    auto t = [&](int d) { return ((B + d - 1) / d) * ((p.n_out + d - 1) / d); };
+    return t(64) >= 2 * 152 ? t(64) : t(32);
+}
+
+// Gradients (into p.g) over B samples, after forward with labels.  da2: buf5, bbuf4; da1: buf6, bbuf5.
+static void backward(ProposalDev &p, int B, cudaStream_t st)
 {
     const int H = p.hidden, I = p.n_in, O = p.n_out;
-    const int64_t nz = (int64_t)B * O;
-    const int nb = blocks_for(nz);
-    // dz (BF16 in bbuf3, FP32 in buf3)
-    bce_kernel<<<nb, 256, 0, st>>>(p.buf[2], Y, p.bbuf[3], p.buf[3], nz, 1.0f / (float)nz, p.loss_parts);
-    gemm(O, H, B, p.bbuf[3], O, true, p.bbuf[2], H, false, p.g + p.off[4], H, 1.0f, 0.0f, st);   // dW3 = dz^T h2
-    colsum_kernel<<<(O + 255) / 256, 256, 0, st>>>(p.buf[3], B, O, p.g + p.off[5]);
-    gemm(B, H, O, p.bbuf[3], O, false, p.wb + p.off[4], H, false, p.buf[4], H, 1.0f, 0.0f, st); // dh2 = dz W3
-    relu_back_kernel<<<blocks_for((int64_t)B * H), 256, 0, st>>>(p.buf[4], p.buf[1], p.bbuf[3], p.buf[5], (int64_t)B * H);
-    gemm(H, H, B, p.bbuf[3], H, true, p.bbuf[1], H, false, p.g + p.off[2], H, 1.0f, 0.0f, st);   // dW2 = da2^T h1
-    colsum_kernel<<<(H + 255) / 256, 256, 0, st>>>(p.buf[5], B, H, p.g + p.off[3]);
-    gemm(B, H, H, p.bbuf[3], H, false, p.wb + p.off[2], H, false, p.buf[4], H, 1.0f, 0.0f, st); // dh1 = da2 W2
-    relu_back_kernel<<<blocks_for((int64_t)B * H), 256, 0, st>>>(p.buf[4], p.buf[0], p.bbuf[3], p.buf[6], (int64_t)B * H);
-    gemm(H, I, B, p.bbuf[3], H, true, p.bbuf[0], I, false, p.g + p.off[0], I, 1.0f, 0.0f, st);   // dW1 = da1^T x
-    colsum_kernel<<<(H + 255) / 256, 256, 0, st>>>(p.buf[6], B, H, p.g + p.off[1]);
-    return nb;
+    JobList q;
+    q.add(product(O, H, B, p.bbuf[3], up8(O), true, p.bbuf[2], H, false, p.g + p.off[4], kEpiStore));             // dW3 = dz^T h2
+    GemmJob g = product(B, H, O, p.bbuf[3], up8(O), false, p.wb + p.off[4], H, false, p.buf[5], kEpiReluBack);    // dh2 = dz W3
+    g.Y = p.buf[1];
+    g.H = p.bbuf[4];
+    q.add(g);
+    q.add(column_sum(p.buf[3], B, O, up8(O), p.g + p.off[5]));
+    q.run(st);
+    q.add(product(H, H, B, p.bbuf[4], H, true, p.bbuf[1], H, false, p.g + p.off[2], kEpiStore));             // dW2 = da2^T h1
+    g = product(B, H, H, p.bbuf[4], H, false, p.wb + p.off[2], H, false, p.buf[6], kEpiReluBack);            // dh1 = da2 W2
+    g.Y = p.buf[0];
+    g.H = p.bbuf[5];
+    q.add(g);
+    q.add(column_sum(p.buf[5], B, H, H, p.g + p.off[3]));
+    q.run(st);
+    q.add(product(H, I, B, p.bbuf[5], H, true, p.bbuf[0], up8(I), false, p.g + p.off[0], kEpiStore));             // dW1 = da1^T x
+    q.add(column_sum(p.buf[6], B, H, H, p.g + p.off[1]));
+    q.run(st);
 }
 
 cudaError_t proposal_forward(ProposalDev &p, const float *X, int n, float *Z, cudaStream_t st)
@@ -334,7 +566,7 @@ cudaError_t proposal_forward(ProposalDev &p, const float *X, int n, float *Z, cu
     }
     for (int s = 0; s < n; s += p.max_batch) {
         const int B = std::min(p.max_batch, n - s);
-        forward(p, X + (size_t)s * p.n_in, B, st);
+        forward(p, X + (size_t)s * p.n_in, nullptr, B, st);
         cudaError_t e = cudaMemcpyAsync(Z + (size_t)s * p.n_out, p.buf[2], sizeof(float) * B * p.n_out,
                                         cudaMemcpyDeviceToDevice, st);
         if (e) return e;
@@ -345,16 +577,12 @@ cudaError_t proposal_forward(ProposalDev &p, const float *X, int n, float *Z, cu
 cudaError_t proposal_grad(ProposalDev &p, const float *X, const float *Y, int n, float *loss, cudaStream_t st)
 {
     if (n > p.max_batch) return cudaErrorInvalidValue;
-    forward(p, X, n, st);
-    const int nb = backward(p, Y, n, st);
-    std::vector<float> parts(nb);
-    cudaError_t e = cudaMemcpyAsync(parts.data(), p.loss_parts, sizeof(float) * nb, cudaMemcpyDeviceToHost, st);
+    forward(p, X, Y, n, st);
+    backward(p, n, st);
+    loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, loss_tiles(p, n), (double)n * p.n_out, p.losses);
+    cudaError_t e = cudaMemcpyAsync(loss, p.losses, sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e) return e;
-    if ((e = cudaStreamSynchronize(st))) return e;
-    double s = 0.0;
-    for (float x : parts) s += x;
-    *loss = (float)(s / ((double)n * p.n_out));
-    return cudaSuccess;
+    return cudaStreamSynchronize(st);
 }
 
 cudaError_t proposal_train(ProposalDev &p, const float *X, const float *Y, int64_t n, int batch, int steps, float lr,
@@ -362,17 +590,26 @@ cudaError_t proposal_train(ProposalDev &p, const float *X, const float *Y, int64
 {
     if (batch > p.max_batch || batch < 1 || n < batch) return cudaErrorInvalidValue;
     int64_t cursor = 0;
+    int done = 0;                                // losses copied out; the device keeps up to kLossSteps
     for (int it = 0; it < steps; ++it) {
         if (cursor + batch > n) cursor = 0;
-        float loss = 0.0f;
-        cudaError_t e = proposal_grad(p, X + cursor * p.n_in, Y + cursor * p.n_out, batch, &loss, st);
-        if (e) return e;
+        forward(p, X + cursor * p.n_in, Y + cursor * p.n_out, batch, st);
+        backward(p, batch, st);
         cursor += batch;
         p.step += 1;
         const float b1 = 0.9f, b2 = 0.999f;
         const float c1 = 1.0f - powf(b1, (float)p.step), c2 = 1.0f - powf(b2, (float)p.step);
         adam_kernel<<<blocks_for(p.n_params), 256, 0, st>>>(p.w, p.g, p.m, p.v, p.wb, p.n_params, lr, b1, b2, 1e-8f, c1, c2);
-        if (losses) losses[it] = loss;
+        cudaError_t e = cudaGetLastError();
+        if (e) return e;
+        if (!losses) continue;
+        loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, loss_tiles(p, batch), (double)batch * p.n_out, p.losses + (it - done));
+        if (it + 1 - done == kLossSteps || it + 1 == steps) {
+            e = cudaMemcpyAsync(losses + done, p.losses, sizeof(float) * (it + 1 - done), cudaMemcpyDeviceToHost, st);
+            if (e) return e;
+            if ((e = cudaStreamSynchronize(st))) return e;
+            done = it + 1;
+        }
     }
     proposal_sync_copies(p, st);
     return cudaGetLastError();

@@ -120,6 +120,48 @@ def test_gradients_match_oracle(am, torch, I, H, O):
         assert rel < 5e-3, (k, rel)
 
 
+@pytest.mark.parametrize("I,H,O,B", [(8, 34, 21, 1), (9, 32, 8, 31), (13, 70, 77, 65), (11, 64, 2049, 600)])
+def test_gradients_at_the_edges_of_the_tiles(am, torch, I, H, O, B):
+    """One sample, one short of a tile, one past it, and a shape whose logits fill the chip with the
+    larger tiles; widths that are no multiple of 8 (element-wise loads) and rows padded to one.  Against
+    the same arithmetic staged exactly: the sums differ by FP32 rounding only, which may move the BF16
+    rounding of an element by one unit (2^-8 at most) in each of two chained products.  The training
+    loop's losses, kept on the device, are those of the gradient call (one sample, a step of no size),
+    also past the 4096 that are kept between copies."""
+    X, Y = _rand_xy(B, I, O, 11)
+    rng = np.random.default_rng(12)
+    with am.Mesher(max_cells=1024, max_neurons=64, max_width=32) as m:
+        m.proposal_init(I, H, O, max_batch=B, seed=5)
+        p = m.proposal_params()
+        m.proposal_set_params(p + 0.05 * rng.normal(size=p.shape).astype(np.float32))
+        prm = unflatten(m.proposal_params(), I, H, O)
+        loss, g = m.proposal_grad(torch.as_tensor(X, device="cuda"), torch.as_tensor(Y, device="cuda"))
+        same = m.proposal_grad(torch.as_tensor(X, device="cuda"), torch.as_tensor(Y, device="cuda"))
+        losses = m.proposal_train(torch.as_tensor(X, device="cuda"), torch.as_tensor(Y, device="cuda"), batch=B,
+                                  steps=4099, lr=1e-30) if B == 1 else None
+    assert same[0] == loss and np.array_equal(same[1], g)
+    if losses is not None:
+        assert len(losses) == 4099 and np.all(losses == np.float32(loss))
+    q = {k: (bf16(torch, v) if k[0] == "W" else v) for k, v in prm.items()}
+    xb = bf16(torch, X)
+    a1 = xb @ q["W1"].T + q["b1"]
+    h1 = bf16(torch, np.maximum(a1, 0))
+    a2 = h1 @ q["W2"].T + q["b2"]
+    h2 = bf16(torch, np.maximum(a2, 0))
+    z = h2 @ q["W3"].T + q["b3"]
+    want = float(np.mean(np.logaddexp(0, z) - Y * z))
+    dz = (1 / (1 + np.exp(-z)) - Y) / Y.size
+    da2 = (bf16(torch, dz) @ q["W3"]) * (a2 > 0)
+    da1 = (bf16(torch, da2) @ q["W2"]) * (a1 > 0)
+    em = {"W3": bf16(torch, dz).T @ h2, "b3": dz.sum(0), "W2": bf16(torch, da2).T @ h1, "b2": da2.sum(0),
+          "W1": bf16(torch, da1).T @ xb, "b1": da1.sum(0)}
+    assert abs(loss - want) <= 2 ** -7 * abs(want), (loss, want)
+    got = unflatten(g, I, H, O)
+    for k in em:
+        rel = np.linalg.norm(got[k] - em[k]) / max(np.linalg.norm(em[k]), 1e-30)
+        assert rel < 2 ** -7, (k, rel)
+
+
 @pytest.mark.parametrize("make,dirs", [(lambda: tiny_net((8, 8), 11), RAY),
                                        (lambda: sphere_net(seed=21, width=32, depth=4, sigma=0.05), RAY)])
 def test_samples_match_oracle(oracle_mod, am, torch, make, dirs):
