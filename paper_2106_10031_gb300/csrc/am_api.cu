@@ -521,6 +521,7 @@ am_status am_load_mlp(am_ctx *ctx, const am_mlp_desc *dsc, int *net_id)
         fhost[i] = h;
         fhost[host.size() + i] = (float)(host[i] - (double)h);
     }
+    const bool finite = std::all_of(fhost.begin(), fhost.end(), [](float f) { return std::isfinite(f); });
     NetHost nh;
     CU(cudaMalloc(&nh.blob, sizeof(double) * host.size()));
     CU(cudaMalloc(&nh.fblob, sizeof(float) * fhost.size()));
@@ -531,6 +532,7 @@ am_status am_load_mlp(am_ctx *ctx, const am_mlp_desc *dsc, int *net_id)
     memset(&nd, 0, sizeof nd);
     nd.L = L;
     nd.N = N;
+    nd.df_finite = finite ? 1 : 0;
     nd.kw = (N + 63) / 64;
     int r0 = 0;
     for (int l = 1; l <= L; ++l) {
@@ -737,6 +739,8 @@ static am_status ensure_seed_cap(am_ctx *ctx, int n)
     return AM_OK;
 }
 
+static int widest(const NetDev &nd) { return *std::max_element(nd.width + 1, nd.width + 1 + nd.L); }
+
 // Dichotomy on n_rays device segments o + t d, t in [0, R] (origins at d_rays, dirs at
 // d_rays + 3 seed_cap), then the push of the new seed cells.  h_points (may be NULL): the
 // seed point of every segment, NaN where it produced none.
@@ -760,6 +764,7 @@ static am_status run_seed(am_ctx *ctx, int net_id, int n_rays, double R, int *n_
     a.seed_ok = ctx->d_seed_ok;
     a.n_new = d_new;
     a.df = ctx->nets[net_id].dev.fp64_only ? 0 : 1;
+    a.width = widest(ctx->nets[net_id].dev);
     launch_seed(a, ctx->stream);
     CU(cudaGetLastError());
     ctx->stats.kernel_launches += 2;
@@ -861,6 +866,7 @@ am_status am_seed_pairs(am_ctx *ctx, int net_id, const double *h_points, int n_p
     p.dirs = ctx->d_rays + 3 * (size_t)ctx->seed_cap;
     p.n_pairs = d_np;
     p.df = ctx->nets[net_id].dev.fp64_only ? 0 : 1;
+    p.width = widest(ctx->nets[net_id].dev);
     launch_pairs(p, ctx->stream);
     CU(cudaGetLastError());
     ctx->stats.kernel_launches += 2;

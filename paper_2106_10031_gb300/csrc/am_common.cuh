@@ -75,6 +75,7 @@ struct NetDev {
     const uint4 *Wf[kMaxLayers + 1];
     const float *wn[kMaxLayers + 1];
     unsigned long long salt;     // per-net hash salt
+    int df_finite;               // 1: every FP32 word of the weight pairs is finite
     int df_ok;                   // 1: the double-float bound stays useful through this net's depth
     double slope;                // hidden activation a (a > 0), slope a (a <= 0); 0 = ReLU
     // residual shortcuts from hidden layers (Sec. 5.1): layer l adds S_l h_{sc_src[l]} (sc_src 0 =

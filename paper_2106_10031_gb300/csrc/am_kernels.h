@@ -102,6 +102,8 @@ void launch_compose(const MarchArgs &a, int mode, const NetDev *net, const unsig
 bool tc_fits(const int *width, int L, int max_n);
 
 struct SeedArgs {
+    int per_block;               // double-float: points per block, set by the launch
+    int width;                   // of the net's widest layer
     const NetDev *nets;
     Arena ar;
     int net;
@@ -137,6 +139,8 @@ void launch_trace(const TraceArgs &a, cudaStream_t st);
 // random-pair sampling (Sec. 4.3.2): F at every sample, then segment r from the r-th negative
 // sample to the r-th positive one, r < min(#neg, #pos, max_pairs)
 struct PairArgs {
+    int per_block;               // double-float: points per block, set by the launch
+    int width;                   // of the net's widest layer
     const NetDev *nets;
     int net;
     int n_points, max_pairs;

@@ -6,6 +6,8 @@
 // ends and is halved until both ends share one activation pattern; inside that cell F is
 // affine along the ray, so the root is t* = t_lo + F_lo / (F_lo - F_hi) (t_hi - t_lo).
 // A second kernel pushes each new seed cell into the active set (hash table + arena).
+#include <algorithm>
+
 #include "am_block.cuh"
 #include "am_kernels.h"
 
@@ -138,16 +140,18 @@ __global__ void __launch_bounds__(kSeedThreads) seed_kernel(SeedArgs a)
 }
 
 // Push the seed cells: allocate an id, write the key, then claim the hash slot with the
-// ref (id, no flip).  A ray landing in an already known cell marks its id dead (-2).
+// ref (id, no flip).  A ray landing in an already known cell marks its id dead (-2).  One warp per ray: the
+// hash is an exclusive or over the key's bits, a word per lane, and lane 0 does the rest (1024 seeds of a
+// 3-[256]x8-1 net take 23 us, with a thread per ray 172).
 __global__ void seed_insert_kernel(SeedArgs a)
 {
-    const int ray = blockIdx.x * blockDim.x + threadIdx.x;
+    const int ray = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (ray >= a.n_rays || a.seed_ok[ray] != 1) return;
     const Arena &ar = a.ar;
     const NetDev &net = a.nets[a.net];
     const unsigned long long *k = a.seed_keys + (size_t)ray * ar.kw;
-    unsigned long long h = net.salt;
-    for (int w = 0; w < ar.kw; ++w) {
+    unsigned long long h = 0ull;
+    for (int w = lane; w < ar.kw; w += 32) {
         unsigned long long x = k[w];
         while (x) {
             const int b = __ffsll((long long)x) - 1;
@@ -155,9 +159,19 @@ __global__ void seed_insert_kernel(SeedArgs a)
             x &= x - 1;
         }
     }
-    const long long id = (long long)atomicAdd(ar.counters + kNCells, 1ull);
-    if (id >= ar.cap) { atomicOr(ar.counters + kStatus, kStCellCap); return; }
-    for (int w = 0; w < ar.kw; ++w) ar.keys[id * ar.kw + w] = k[w];
+    for (int o = 16; o > 0; o >>= 1) h ^= __shfl_xor_sync(0xffffffffu, h, o);
+    h ^= net.salt;
+    long long id = 0;
+    if (lane == 0) id = (long long)atomicAdd(ar.counters + kNCells, 1ull);
+    id = __shfl_sync(0xffffffffu, id, 0);
+    if (id >= ar.cap) {
+        if (lane == 0) atomicOr(ar.counters + kStatus, kStCellCap);
+        return;
+    }
+    for (int w = lane; w < ar.kw; w += 32) ar.keys[id * ar.kw + w] = k[w];
+    __threadfence();
+    __syncwarp();
+    if (lane != 0) return;
     ar.net[id] = a.net;
     ar.hash[id] = h;
     ar.nverts[id] = -1;
@@ -288,48 +302,64 @@ __global__ void __launch_bounds__(kSeedThreads) trace_kernel(TraceArgs a)
 }
 
 // ------------------------------------------------------------------------------------------
-// The same forward pass in double-float arithmetic, kDfPts points per block, for nets without
+// The same forward pass in double-float arithmetic, up to kDfPts points per block, for nets without
 // hidden shortcuts, pooling or leaky units: the pairs (hi, lo) of FP32 words carry about 44 bits
 // (the product of two pairs split exactly by an FMA, sums by TwoSum), so F and the pattern bits
-// agree with an FP64 evaluation wherever they are not within ~1e-12 of zero.  Each weight pair
-// is read once per block for all its points, and the arithmetic runs on the FP32 pipes (this
-// part's FP64 pipe is 1/64 of them).
+// agree with an FP64 evaluation wherever they are not within ~1e-12 of zero.  The arithmetic runs on the
+// FP32 pipes (this part's FP64 pipe is 1/64 of them), 12 instructions per product, which bound it.
+//
+// A warp takes one point and 32 units, and only that point's active inputs (about half of them: the
+// others are zero, and a product with zero changes no bit of the sum), from a list of (hi, lo, offset of
+// the weights) in shared memory; warps of the block's other points run beside it on the same 32 units and
+// find the weights in the L1.  With eight points per thread, all inputs and 8 warps per SM, the 16384
+// samples of a 3-[256]x8-1 net took 3.99 ms and the dichotomy of its 1024 segments 8.64; 3.09 and 3.48 now.
 
-constexpr int kDfPts = 8;                  // points per block
-constexpr int kDfW = kSeedThreads / 32;
+constexpr int kDfPts = 4;                  // points per block, at most
+constexpr int kDfThreads = 512;            // threads per block, at most
+constexpr int kDfSums = kSeedThreads / 32; // partial sums of F: units 32 v + lane + kSeedThreads i in sum v
 
 __host__ __device__ inline int df_seed_smem_bytes(int max_n, int max_w)
 {
-    const int words = (max_n + 31) / 32;
-    return 2 * max_w * 2 * kDfPts * (int)sizeof(float)           // two layers' outputs: [j][hi x 8 | lo x 8]
+    const int words = (max_n + 31) / 32, chunks = (max_w + 31) / 32;
+    return kDfPts * (max_w + 8) * (int)sizeof(float4)            // active inputs
+           + kDfPts * max_w * (int)sizeof(float2)                // a layer's outputs
+           + kDfPts * (chunks + 1) * (int)sizeof(unsigned)       // its active units, and the list's length
            + 3 * kDfPts * words * (int)sizeof(unsigned)          // patterns: the bracket's ends, the midpoint
            + kDfPts * 8 * (int)sizeof(float)                     // the points as pairs
-           + kDfPts * kDfW * 2 * (int)sizeof(float)              // partial sums of F
+           + kDfPts * kDfSums * (int)sizeof(float2)              // partial sums of F
            + kDfPts * (int)sizeof(double) + 64;
 }
 
 struct DfSm {
-    float *h[2];                // layer outputs, element (j, p): hi at [16 j + p], lo at [16 j + 8 + p]
+    float4 *list;               // point p at [p (max_w + 8)]: active inputs (hi, lo, offset of their weights)
+    float2 *z;                  // point p at [p max_w]: the last layer's outputs, zero where inactive
+    float2 *red;
+    unsigned *on;               // point p at [p chunks]: the layer's active units
+    int *cnt;                   // entries of p's list, a multiple of eight
     unsigned *blo, *bhi, *bm;   // patterns, point p at [p words]
     float *xp;                  // point p: [xh, yh, zh, xl, yl, zl] at [8 p]
-    float *red;
     double *F;
+    int max_w, chunks;
 };
 
 __device__ inline DfSm df_carve(unsigned char *base, int max_n, int max_w)
 {
     const int words = (max_n + 31) / 32;
     DfSm s;
-    float *f = reinterpret_cast<float *>(base);
-    s.h[0] = f;
-    s.h[1] = f + 16 * max_w;
-    unsigned *u = reinterpret_cast<unsigned *>(f + 32 * max_w);
+    s.max_w = max_w;
+    s.chunks = (max_w + 31) / 32;
+    s.list = reinterpret_cast<float4 *>(base);
+    s.z = reinterpret_cast<float2 *>(s.list + kDfPts * (max_w + 8));
+    s.red = s.z + kDfPts * max_w;
+    unsigned *u = reinterpret_cast<unsigned *>(s.red + kDfPts * kDfSums);
+    s.on = u;
+    s.cnt = reinterpret_cast<int *>(u + kDfPts * s.chunks);
+    u += kDfPts * (s.chunks + 1);
     s.blo = u;
     s.bhi = u + kDfPts * words;
     s.bm = u + 2 * kDfPts * words;
     s.xp = reinterpret_cast<float *>(u + 3 * kDfPts * words);
-    s.red = s.xp + 8 * kDfPts;
-    s.F = reinterpret_cast<double *>(((uintptr_t)(s.red + 2 * kDfW * kDfPts) + 15) & ~(uintptr_t)15);
+    s.F = reinterpret_cast<double *>(((uintptr_t)(s.xp + 8 * kDfPts) + 15) & ~(uintptr_t)15);
     return s;
 }
 
@@ -367,121 +397,180 @@ __device__ __forceinline__ void df_set_point(const DfSm &s, int p, const double 
     }
 }
 
-// F at the block's first NP points (s.xp; the caller sets each of them, unused ones anywhere
-// finite) into s.F, and their patterns (Def. 2) into bits[p words].  Every thread calls it.
-// NP is 8, 4, 2 or 1: a dichotomy whose other rays are done evaluates only what is left.
-template <int NP>
-__device__ void df_forward_batch(const NetDev &net, const DfSm &s, unsigned *bits)
+// Layer l of the block's first n points, U units a lane: 32 U units and one point per warp at a time.
+template <int U>
+__device__ __forceinline__ void df_layer(const NetDev &net, const DfSm &s, unsigned *bits, int n, int l)
 {
-    static_assert(NP == 1 || NP == 2 || NP == 4 || NP == 8, "points per pass");
-    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wid = tid >> 5;
-    const int words = (net.N + 31) / 32;
-    for (int w = tid; w < NP * words; w += T) bits[w] = 0u;
-    __syncthreads();
-    for (int l = 1; l <= net.L; ++l) {
-        const int nl = net.width[l], np = l > 1 ? net.width[l - 1] : 0, rl = net.row0[l];
-        const float *Ch = net.Clhi[l], *Cc = net.Cllo[l];
-        const float *Ah = net.AThi[l], *Al = net.ATlo[l];
-        const float *ph = s.h[(l - 1) & 1];
-        float *out = s.h[l & 1];
-        for (int k = tid; k < nl; k += T) {
-            float sh[NP], sl[NP];
-            const float bh = Ch[4 * k + 3], bl = Cc[4 * k + 3];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int words = (net.N + 31) / 32, nl = net.width[l], rl = net.row0[l], chunks = (nl + 32 * U - 1) / (32 * U);
+    const float *Ch = net.Clhi[l], *Cc = net.Cllo[l];
+#pragma unroll 1
+    for (int item = wid; item < n * chunks; item += warps) {
+        const int p = item % n, k0 = item / n * (32 * U);
+        float sh[U], sl[U];
+        const float *Ah[U], *Al[U];
 #pragma unroll
-            for (int p = 0; p < NP; ++p) { sh[p] = bh; sl[p] = bl; }
+        for (int e = 0; e < U; ++e) {
+            const int k = min(k0 + 32 * e + lane, nl - 1);
+            Ah[e] = l > 1 ? net.AThi[l] + k : nullptr;
+            Al[e] = l > 1 ? net.ATlo[l] + k : nullptr;
+            sh[e] = Ch[4 * k + 3];
+            sl[e] = Cc[4 * k + 3];
+#pragma unroll
             for (int c = 0; c < 3; ++c) {                // the input columns (layer 1, and skip layers)
                 const float wh = Ch[4 * k + c], wl = Cc[4 * k + c];
                 if (wh == 0.0f && wl == 0.0f) continue;
-#pragma unroll
-                for (int p = 0; p < NP; ++p) dfs_fma(sh[p], sl[p], wh, wl, s.xp[8 * p + c], s.xp[8 * p + 3 + c]);
+                dfs_fma(sh[e], sl[e], wh, wl, s.xp[8 * p + c], s.xp[8 * p + 3 + c]);
             }
-            for (int j = 0; j < np; ++j) {
-                const float ah = __ldg(Ah + (size_t)j * nl + k), al = __ldg(Al + (size_t)j * nl + k);
-                float zh[NP], zl[NP];
-                if constexpr (NP >= 4) {
-                    const float4 *hj = reinterpret_cast<const float4 *>(ph + 16 * j);
+        }
+        const int m = l > 1 ? s.cnt[p] : 0;
+        if (m > 0) {
+            // B inputs at a time, the next B's weights on their way (the lists end on a multiple of 8)
+            constexpr int B = 4 / U;
+            const float4 *in = s.list + p * (s.max_w + 8);
+            struct Ahead { float2 z[B]; float h[B][U], lo[B][U]; } a, b;
+            auto fetch = [&](Ahead &q, int t) {
 #pragma unroll
-                    for (int g = 0; g < NP / 4; ++g) {
-                        const float4 h4 = hj[g], l4 = hj[2 + g];
-                        zh[4 * g] = h4.x; zh[4 * g + 1] = h4.y; zh[4 * g + 2] = h4.z; zh[4 * g + 3] = h4.w;
-                        zl[4 * g] = l4.x; zl[4 * g + 1] = l4.y; zl[4 * g + 2] = l4.z; zl[4 * g + 3] = l4.w;
+                for (int u = 0; u < B; ++u) {
+                    const float4 v = in[t + u];
+                    q.z[u] = make_float2(v.x, v.y);
+#pragma unroll
+                    for (int e = 0; e < U; ++e) {
+                        q.h[u][e] = __ldg(Ah[e] + __float_as_int(v.z));
+                        q.lo[u][e] = __ldg(Al[e] + __float_as_int(v.z));
                     }
-                } else {
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) { zh[p] = ph[16 * j + p]; zl[p] = ph[16 * j + 8 + p]; }
                 }
+            };
+            auto multiply = [&](const Ahead &q) {
 #pragma unroll
-                for (int p = 0; p < NP; ++p) dfs_fma(sh[p], sl[p], ah, al, zh[p], zl[p]);
+                for (int u = 0; u < B; ++u)
+#pragma unroll
+                    for (int e = 0; e < U; ++e) dfs_fma(sh[e], sl[e], q.h[u][e], q.lo[u][e], q.z[u].x, q.z[u].y);
+            };
+            fetch(a, 0);
+#pragma unroll 1
+            for (int t = 0; t < m; t += 2 * B) {
+                fetch(b, t + B);
+                multiply(a);
+                if (t + 2 * B < m) fetch(a, t + 2 * B);
+                multiply(b);
             }
+        }
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const float t = __fadd_rn(sh[p], sl[p]);       // renormalise: sign(pair) = sign(hi)
-                const float lo = __fsub_rn(sl[p], __fsub_rn(t, sh[p]));
-                const bool act = t > 0.0f;
-                out[16 * k + p] = act ? t : 0.0f;
-                out[16 * k + 8 + p] = act ? lo : 0.0f;
-                if (act) atomicOr(bits + p * words + ((rl + k) >> 5), 1u << ((rl + k) & 31));
+        for (int e = 0; e < U; ++e) {
+            const int k = k0 + 32 * e + lane;
+            const float t = __fadd_rn(sh[e], sl[e]);       // renormalise: sign(pair) = sign(hi)
+            const float lo = __fsub_rn(sl[e], __fsub_rn(t, sh[e]));
+            const bool act = k < nl && t > 0.0f;
+            if (k < nl) s.z[p * s.max_w + k] = act ? make_float2(t, lo) : make_float2(0.0f, 0.0f);
+            const unsigned b = __ballot_sync(0xffffffffu, act);
+            if (lane == 0 && k < nl) {
+                s.on[p * s.chunks + (k >> 5)] = b;
+                const int bit = rl + k, sft = bit & 31;
+                unsigned *o = bits + p * words + (bit >> 5);
+                if (b << sft) atomicOr(o, b << sft);
+                if (sft && (b >> (32 - sft))) atomicOr(o + 1, b >> (32 - sft));
+            }
+        }
+    }
+}
+
+// F at the block's first n (1 to kDfPts) points (s.xp, set by the caller) into s.F, and their patterns
+// (Def. 2) into bits[p words].  Every thread calls it.
+__device__ void df_forward(const NetDev &net, const DfSm &s, unsigned *bits, int n)
+{
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wid = tid >> 5, warps = T >> 5;
+    const int words = (net.N + 31) / 32, L = net.L;
+    const bool all = !net.df_finite;               // a product of a zero with a weight out of range is no zero
+    for (int w = tid; w < n * words; w += T) bits[w] = 0u;
+    __syncthreads();
+#pragma unroll 1
+    for (int l = 1; l <= L; ++l) {
+        // two units a lane share the point's input and most of the address arithmetic (16 instructions per
+        // product against 20: 3.27 ms for the samples above with one unit), when that leaves three quarters of the warps one item at least
+        const int nl = net.width[l], chunks = (nl + 31) >> 5;
+        if (nl > 32 && n * ((nl + 63) >> 6) >= 3 * (warps >> 2)) df_layer<2>(net, s, bits, n, l);
+        else df_layer<1>(net, s, bits, n, l);
+        __syncthreads();
+        if (l == L) break;
+        // the active outputs, in order, as the next layer's inputs
+        const int n2 = net.width[l + 1];
+        for (int item = wid; item < n * 4; item += warps) {
+            const int p = item >> 2, q = item & 3;
+            float4 *out = s.list + p * (s.max_w + 8);
+            int at = 0;
+            for (int c = 0; c < chunks; ++c) {
+                unsigned b = s.on[p * s.chunks + c];
+                if (all) b = 32 * c + 32 <= nl ? full : (1u << (nl - 32 * c)) - 1u;
+                if ((c & 3) == q && ((b >> lane) & 1u)) {
+                    const int k = 32 * c + lane;
+                    const float2 z = s.z[p * s.max_w + k];
+                    out[at + __popc(b & ((1u << lane) - 1u))] = make_float4(z.x, z.y, __int_as_float(k * n2), 0.0f);
+                }
+                at += __popc(b);
+            }
+            if (q == 0) {                                  // zeros to a multiple of eight (weights of unit 0)
+                const int m = (at + 7) & ~7;
+                if (lane < m - at) out[at + lane] = make_float4(0.0f, 0.0f, __int_as_float(0), 0.0f);
+                if (lane == 0) s.cnt[p] = m;
             }
         }
         __syncthreads();
     }
-    const int nL = net.width[net.L];
-    const float *hL = s.h[net.L & 1];
-    float fh[NP], fl[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) { fh[p] = 0.0f; fl[p] = 0.0f; }
-    for (int k = tid; k < nL; k += T) {
-        const float wh = net.w_out_hi[k], wl = net.w_out_lo[k];
-#pragma unroll
-        for (int p = 0; p < NP; ++p) dfs_fma(fh[p], fl[p], wh, wl, hL[16 * k + p], hL[16 * k + 8 + p]);
-    }
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, fh[p], o), ol = __shfl_xor_sync(0xffffffffu, fl[p], o);
-            dfs_add(fh[p], fl[p], oh, ol);
+    const int nL = net.width[L];
+    for (int item = wid; item < n * kDfSums; item += warps) {
+        const int p = item / kDfSums, v = item % kDfSums;
+        float fh = 0.0f, fl = 0.0f;
+        for (int k = 32 * v + lane; k < nL; k += kSeedThreads) {
+            const float2 z = s.z[p * s.max_w + k];
+            dfs_fma(fh, fl, net.w_out_hi[k], net.w_out_lo[k], z.x, z.y);
         }
-        if (lane == 0) { s.red[2 * (p * kDfW + wid)] = fh[p]; s.red[2 * (p * kDfW + wid) + 1] = fl[p]; }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_xor_sync(full, fh, o), ol = __shfl_xor_sync(full, fl, o);
+            dfs_add(fh, fl, oh, ol);
+        }
+        if (lane == 0) s.red[item] = make_float2(fh, fl);
     }
     __syncthreads();
-    if (tid < NP) {
+    if (tid < n) {
         double F = net.b_out;
-        for (int w = 0; w < T / 32; ++w) F += (double)s.red[2 * (tid * kDfW + w)] + (double)s.red[2 * (tid * kDfW + w) + 1];
+        for (int v = 0; v < kDfSums; ++v) {
+            const float2 f = s.red[tid * kDfSums + v];
+            F += (double)f.x + (double)f.y;
+        }
         s.F[tid] = F;
     }
     __syncthreads();
 }
 
-// the forward pass of the first n (1..8) points, in the smallest batch that holds them
-__device__ void df_forward_n(const NetDev &net, const DfSm &s, unsigned *bits, int n)
-{
-    if (n > 4) df_forward_batch<8>(net, s, bits);
-    else if (n > 2) df_forward_batch<4>(net, s, bits);
-    else if (n > 1) df_forward_batch<2>(net, s, bits);
-    else df_forward_batch<1>(net, s, bits);
-}
+// Points per block for n of them: one per SM before they share weights.  Threads: a warp for every 32 units
+// and point, up to kDfThreads (1024 pairs of a 3-[24]x3-1 net: 334 us, 397 with 512 threads).
+static int df_points(int n) { return std::min(kDfPts, std::max(1, (n + 151) / 152)); }
+static int df_threads(int width) { return std::min(kDfThreads, 32 * kDfPts * ((width + 31) / 32)); }
 
-// F at every sample point (random-pair trigger, Sec. 4.3.2), kDfPts points per block
-__global__ void __launch_bounds__(kSeedThreads) sample_eval_df_kernel(PairArgs a)
+// F at every sample point (random-pair trigger, Sec. 4.3.2), a.per_block points per block
+__global__ void __launch_bounds__(kDfThreads, 2) sample_eval_df_kernel(PairArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const NetDev &net = a.nets[a.net];
     const DfSm s = df_carve(smem, a.max_n, a.max_w);
-    const int i0 = blockIdx.x * kDfPts, P = min(kDfPts, a.n_points - i0);
+    const int i0 = blockIdx.x * a.per_block, P = min(a.per_block, a.n_points - i0);
     if (threadIdx.x < kDfPts) {
         const int i = i0 + (threadIdx.x < P ? threadIdx.x : 0);
         const double x[3] = {a.points[3 * i], a.points[3 * i + 1], a.points[3 * i + 2]};
         df_set_point(s, threadIdx.x, x);
     }
     __syncthreads();
-    df_forward_n(net, s, s.bm, P);
+    df_forward(net, s, s.bm, P);
     if (threadIdx.x < P) a.F[i0 + threadIdx.x] = s.F[threadIdx.x];
 }
 
-// The dichotomy of seed_kernel for kDfPts rays per block, in double-float: one batched forward
+// The dichotomy of seed_kernel for a.per_block rays per block, in double-float: one batched forward
 // pass per halving step of the block's rays that still bracket more than one cell, packed into
 // the first slots so that a step with fewer rays left evaluates fewer points.
-__global__ void __launch_bounds__(kSeedThreads) seed_df_kernel(SeedArgs a)
+__global__ void __launch_bounds__(kDfThreads, 2) seed_df_kernel(SeedArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double tlo[kDfPts], thi[kDfPts], flo[kDfPts], fhi[kDfPts], tm[kDfPts];
@@ -489,7 +578,7 @@ __global__ void __launch_bounds__(kSeedThreads) seed_df_kernel(SeedArgs a)
     const NetDev &net = a.nets[a.net];
     const DfSm s = df_carve(smem, a.max_n, a.max_w);
     const int tid = threadIdx.x, words = (net.N + 31) / 32;
-    const int r0 = blockIdx.x * kDfPts, P = min(kDfPts, a.n_rays - r0);
+    const int r0 = blockIdx.x * a.per_block, P = min(a.per_block, a.n_rays - r0);
     auto point = [&](int q, int p, double t) {          // slot q: ray p's point at t (rays past P: ray 0)
         const int r = r0 + (p < P ? p : 0);
         const double x[3] = {a.origins[3 * r] + t * a.dirs[3 * r], a.origins[3 * r + 1] + t * a.dirs[3 * r + 1],
@@ -498,10 +587,10 @@ __global__ void __launch_bounds__(kSeedThreads) seed_df_kernel(SeedArgs a)
     };
     if (tid < kDfPts) { tlo[tid] = 0.0; thi[tid] = a.R; point(tid, tid, 0.0); }
     __syncthreads();
-    df_forward_n(net, s, s.blo, P);
+    df_forward(net, s, s.blo, P);
     if (tid < kDfPts) { flo[tid] = s.F[tid]; point(tid, tid, a.R); }
     __syncthreads();
-    df_forward_n(net, s, s.bhi, P);
+    df_forward(net, s, s.bhi, P);
     if (tid < kDfPts) {
         fhi[tid] = s.F[tid];
         const double f0 = flo[tid], f1 = fhi[tid];
@@ -536,7 +625,7 @@ __global__ void __launch_bounds__(kSeedThreads) seed_df_kernel(SeedArgs a)
             point(tid, p, tm[p]);
         }
         __syncthreads();
-        df_forward_n(net, s, s.bm, nact);
+        df_forward(net, s, s.bm, nact);
         if (tid < nact) {
             const int p = slot_ray[tid];
             const double fm = s.F[tid];
@@ -647,23 +736,28 @@ void launch_trace(const TraceArgs &a, cudaStream_t st)
     trace_kernel<<<a.n, kSeedThreads, seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
 }
 
-void launch_pairs(const PairArgs &a, cudaStream_t st)
+void launch_pairs(const PairArgs &args, cudaStream_t st)
 {
+    PairArgs a = args;
+    a.per_block = df_points(a.n_points);
     if (a.df)
-        sample_eval_df_kernel<<<(a.n_points + kDfPts - 1) / kDfPts, kSeedThreads, df_seed_smem_bytes(a.max_n, a.max_w),
-                                st>>>(a);
+        sample_eval_df_kernel<<<(a.n_points + a.per_block - 1) / a.per_block, df_threads(a.width),
+                                df_seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
     else
         sample_eval_kernel<<<a.n_points, kSeedThreads, seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
     pair_build_kernel<<<1, kPairThreads, 0, st>>>(a);
 }
 
-void launch_seed(const SeedArgs &a, cudaStream_t st)
+void launch_seed(const SeedArgs &args, cudaStream_t st)
 {
+    SeedArgs a = args;
+    a.per_block = df_points(a.n_rays);
     if (a.df)
-        seed_df_kernel<<<(a.n_rays + kDfPts - 1) / kDfPts, kSeedThreads, df_seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
+        seed_df_kernel<<<(a.n_rays + a.per_block - 1) / a.per_block, df_threads(a.width),
+                         df_seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
     else
         seed_kernel<<<a.n_rays, kSeedThreads, seed_smem_bytes(a.max_n, a.max_w), st>>>(a);
-    seed_insert_kernel<<<(a.n_rays + 127) / 128, 128, 0, st>>>(a);
+    seed_insert_kernel<<<(a.n_rays + 3) / 4, 128, 0, st>>>(a);
 }
 
 }  // namespace am

@@ -3,7 +3,7 @@ SDF (Sec. 4.3.1) and the random-pair dichotomy (Sec. 4.3.2).  Needs a GPU."""
 import numpy as np
 import pytest
 
-from synth import polytope_max_of_planes, sphere_net, tiny_net, trigger_points
+from synth import decoder_net, polytope_max_of_planes, sphere_net, tiny_net, trigger_points
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -110,3 +110,39 @@ def test_trigger_edge_cases(am):
         with pytest.raises(am.AMError) as e:
             m.seed_sphere_trace(nid, [[0.3, 0.2, 0.1]])
         assert e.value.status == 5
+
+
+@pytest.mark.parametrize("make,n_pairs,box", [
+    (lambda: sphere_net(seed=21, width=31, depth=3, sigma=0.05), 1, 0.5),
+    (lambda: sphere_net(seed=21, width=65, depth=3, sigma=0.05), 5, 0.5),
+    (lambda: tiny_net((129, 40, 7), 7), 610, 0.5),
+    (lambda: sphere_net(seed=21, width=256, depth=3, sigma=0.01), 157, 0.5),
+    (lambda: decoder_net(width=40, depth=5, latent_dim=9, skip_layer=3, seed=7, sigma=0.05), 305, 1.2),
+])
+def test_pairs_at_the_edges_of_the_warps(oracle_mod, am, make, n_pairs, box):
+    # widths around 32 and 64 units, one to four points per block with a ragged last one, one and two units a
+    # lane, a skip layer: pairs of 1e-13 accuracy, so the seed points are the oracle's to 1e-9
+    mlp = make()
+    net = oracle_mod.OracleNet(mlp)
+    pts = trigger_points(6 * n_pairs + 7, seed=21, box=box)
+    seeds = oracle_mod.seed_pairs(net, pts, n_pairs)
+    assert len(seeds) == n_pairs
+    live = [s for s in seeds if s is not None]
+    with am.Mesher(max_cells=1 << 16, max_neurons=1024, max_width=256) as m:
+        nid = m.load_mlp(mlp)
+        got_pairs, n_new, got = m.seed_pairs(nid, pts, n_pairs)
+        assert got_pairs == len(seeds)
+        assert n_new == len({k for k, _ in live})
+        _check_points(got, _ref_points(seeds, got_pairs))
+
+
+def test_weights_beyond_single_range_find_no_seed(am):
+    # such a weight has no (hi, lo) pair, so F is no number, also where the weight's input is inactive
+    mlp = tiny_net((8, 8), 1, sigma=0.3)
+    pts = trigger_points(300, seed=7, box=1.5)
+    mlp.biases[0][3] = -100.0
+    mlp.weights[1][:, 3] = 1e39
+    with am.Mesher(max_cells=1 << 12, max_neurons=64, max_width=64) as m:
+        nid = m.load_mlp(mlp)
+        with pytest.raises(am.AMError):
+            m.seed_pairs(nid, pts, 48)
