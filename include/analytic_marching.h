@@ -193,10 +193,10 @@ typedef struct {
     int64_t close_calls;      /* mixed precision: sign tests re-evaluated in FP64 */
     int64_t fixups;           /* faces whose candidate polygon the all-row check corrected */
     int64_t cuts;             /* half-plane cuts applied to face polygons (candidates + corrections) */
-    int64_t phase_cycles[10]; /* SM cycles summed over cells per phase (compose, set-up, candidate
-                                 sort, candidate clip, FP64 vertices, check, emit, march, waiting
-                                 for work, spare); only filled by a build with -DAM_PHASE_TIMERS,
-                                 zero otherwise */
+    int64_t phase_cycles[10]; /* SM cycles summed over cells per phase (compose, candidate lines,
+                                 candidate sort, edge intervals, ring and FP64 vertices, check, emit,
+                                 push, waiting for work, sequential clip); only filled by a build with
+                                 -DAM_PHASE_TIMERS, zero otherwise */
     double ms_compose;        /* AM_PREC_SLICED march: device time of the tensor-core compose launches */
     double ms_clip;           /* AM_PREC_SLICED march: device time of the clip launches reading those rows */
     double ms_proposal;       /* AM_PREC_SLICED march with AM_CAND_LEARNED: device time of the proposal's

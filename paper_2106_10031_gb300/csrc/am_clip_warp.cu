@@ -83,41 +83,27 @@ struct WRows {
             r[3] = k < N + kBoxPlanes ? (double)h.w - (double)box_lo : (double)h.w;
         }
     }
-    __device__ __forceinline__ void f32(int k, float *r) const
-    {
-        const float4 h = hi(k);
-        r[0] = h.x; r[1] = h.y; r[2] = h.z; r[3] = h.w;
-    }
 };
 
-template <class R>
-__device__ __forceinline__ R wpdist(const R *r, R ri, const R *v)
+__device__ __forceinline__ double wpdist(const double *r, double ri, const double *v)
 {
     return (r[0] * v[0] + r[1] * v[1] + r[2] * v[2] + r[3]) * ri;
-}
-
-template <class R>
-__device__ __forceinline__ void wrow(const WRows &rv, int k, R *r)
-{
-    if constexpr (sizeof(R) == 8) rv.f64(k, r);
-    else rv.f32(k, r);
 }
 
 // One cut of the polygon P[buf] (m vertices) by row k, the warp's lanes over the vertices: a
 // vertex is cut off when its distance from row k's plane exceeds tol; the two new vertices are
 // solved from their planes and the face plane aF.  Returns the new count (0 = empty, -1 =
 // inconsistent or beyond kWPoly); *swapped: the result went to buffer buf ^ 1.
-template <class R>
-__device__ int wcut(WarpSh &S, R (*P)[kWPoly][3], int m, int buf, int k, R tol, const R *aF, const WRows &rv,
+__device__ int wcut(WarpSh &S, double (*P)[kWPoly][3], int m, int buf, int k, double tol, const double *aF, const WRows &rv,
                     bool *swapped)
 {
     const int lane = threadIdx.x & 31;
     *swapped = false;
-    R rk[4];
-    wrow<R>(rv, k, rk);
-    const R rn = sqrt(rk[0] * rk[0] + rk[1] * rk[1] + rk[2] * rk[2]);
-    if (rn == R(0)) return m;
-    const R ri = R(1) / rn;
+    double rk[4];
+    rv.f64(k, rk);
+    const double rn = sqrt(rk[0] * rk[0] + rk[1] * rk[1] + rk[2] * rk[2]);
+    if (rn == 0.0) return m;
+    const double ri = 1.0 / rn;
     const bool o0 = lane < m && wpdist(rk, ri, P[buf][lane]) > tol;
     const bool o1 = lane + 32 < m && wpdist(rk, ri, P[buf][lane + 32]) > tol;
     const unsigned long long out = (unsigned long long)__ballot_sync(0xffffffffu, o0) |
@@ -150,10 +136,10 @@ __device__ int wcut(WarpSh &S, R (*P)[kWPoly][3], int m, int buf, int k, R tol, 
     }
     bool ok = true;
     if (lane < 2) {
-        R pa[4], pb[4], v[3];
-        wrow<R>(rv, lane == 0 ? ea : k, pa);
-        wrow<R>(rv, lane == 0 ? k : eb, pb);
-        ok = solve3<R>(pa, pb, aF, v, nullptr);
+        double pa[4], pb[4], v[3];
+        rv.f64(lane == 0 ? ea : k, pa);
+        rv.f64(lane == 0 ? k : eb, pb);
+        ok = solve3<double>(pa, pb, aF, v, nullptr);
         P[nb][nin + lane][0] = v[0]; P[nb][nin + lane][1] = v[1]; P[nb][nin + lane][2] = v[2];
         S.pe[nb][nin + lane] = lane == 0 ? k : eb;
     }
@@ -183,12 +169,6 @@ __device__ bool wfinal(WarpSh &S, int m, int buf, const WRows &rv)
     ok = __all_sync(0xffffffffu, ok);
     __syncwarp();
     return ok;
-}
-
-__device__ __forceinline__ unsigned order_key(float d)
-{
-    const unsigned du = __float_as_uint(d);
-    return (du & 0x80000000u) ? ~du : (du | 0x80000000u);
 }
 
 // the cell's key as 32-bit words in the warp's shared memory (pushes copy it)
@@ -360,7 +340,7 @@ __device__ bool wcheck(const MarchArgs &a, WarpSh &S, const WRows &rv, int N, in
         if (rounds + 1 >= kWMaxFix) { fallback = true; break; }
         for (int t = 0; t < nviol && m > 0; ++t) {
             bool sw;
-            const int nm = wcut<double>(S, S.pv, m, buf, S.viol[t], 0.0, S.aF, rv, &sw);
+            const int nm = wcut(S, S.pv, m, buf, S.viol[t], 0.0, S.aF, rv, &sw);
             if (nm < 0) { fallback = true; break; }
             if (sw) buf ^= 1;
             m = nm;
