@@ -96,6 +96,27 @@ __device__ __forceinline__ unsigned long long child_word(unsigned long long x, i
     return x;
 }
 
+// Twice the smallest kept area (1e-24 box^2) from above, for area_clear (in FP32: the FP64 pipe is a scarce one)
+__device__ __forceinline__ float area_min(float box) { return fmaxf(2e-24f * box * box * 1.0001f, 1e-30f); }
+
+// Whether a face is larger than the smallest kept one beyond every rounding: the triangle of three of its
+// vertices lies in it.  p, q, r are the vertices in FP32, each coordinate within u |v|_inf (u = 2^-24, X the
+// largest coordinate) of the FP64 one that the area rule reads, so a side's coordinate is off by
+// d <= 4.1 u X, a component of the cross product by d (|a|_1 + |b|_1) + 2 d^2 and its own rounding, at most
+// 3 u X (|a|_1 + |b|_1): below 12 u X (|a|_1 + |b|_1) wherever the component exceeds that (2 d^2 = 34 u^2 X^2
+// matters only for sides of that size, whose product is smaller).  False: FP64 decides, from the FP64 vertices.
+// Nothing here is a length of its own, so it holds in a box of any size; three vertices cost less than the
+// sum over all edges (no reduction over the lanes).
+__device__ __forceinline__ bool area_clear(const float4 p, const float4 q, const float4 r, float amin)
+{
+    const float ax = q.x - p.x, ay = q.y - p.y, az = q.z - p.z, bx = r.x - p.x, by = r.y - p.y, bz = r.z - p.z;
+    const float c = fmaxf(fabsf(ay * bz - az * by), fmaxf(fabsf(az * bx - ax * bz), fabsf(ax * by - ay * bx)));
+    const float s = fabsf(ax) + fabsf(ay) + fabsf(az) + fabsf(bx) + fabsf(by) + fabsf(bz);
+    const float X = fmaxf(fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(p.z), fabsf(q.x))),
+                          fmaxf(fmaxf(fabsf(q.y), fabsf(q.z)), fmaxf(fmaxf(fabsf(r.x), fabsf(r.y)), fabsf(r.z))));
+    return c > fmaf(12.0f * 5.9604645e-8f * X, s, amin);
+}
+
 // the words of two keys a and b crossed at fa and fb, compared (max-pooled nets; out of line)
 static __device__ __noinline__ unsigned long long pooled_diff(unsigned long long a, unsigned long long b, int w, unsigned fa,
                                                        unsigned fb, int pool0, int pool1)

@@ -850,11 +850,7 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
             continue;
         }
         // ---- a6 emit: the face's area in FP32 where that is clear of every rounding, else in FP64
-        const float nxv = __shfl_sync(FULL, vx, lane + 1 < m ? lane + 1 : 0), nyv = __shfl_sync(FULL, vy, lane + 1 < m ? lane + 1 : 0);
-        float area = lane < m ? vx * nyv - nxv * vy - 1e-5f * (fabsf(vx * nyv) + fabsf(nxv * vy)) : 0.0f;
-#pragma unroll 1
-        for (int o = 16; o > 0; o >>= 1) area += __shfl_xor_sync(FULL, area, o);
-        int emit = area > 1e-11f || clip_area(S, m, a.box) ? m : 0;
+        int emit = area_clear(S.vf[0], S.vf[m / 3], S.vf[2 * m / 3], area_min(a.box_hi)) || clip_area(S, m, a.box) ? m : 0;
         if (emit > ar.maxv) {
             if (lane == 0) atomicOr(ar.counters + kStatus, kStFaceVerts);
             emit = 0;

@@ -1140,14 +1140,13 @@ __device__ __forceinline__ float4 row32(const Sh &s, int k)
 
 // Warp 0: the ring of the lines' intervals (s.seg).  A line carries an edge when the part of it
 // inside all others is not empty; the line that ends an edge carries the next one.  Writes the
-// edge planes s.pe[0][0 .. m) counter-clockwise and the area flag s.si[6] (1: clearly above the
-// smallest kept area, 2: FP64 decides); returns m, or 0 when the edges do not close into one ring.
+// edge planes s.pe[0][0 .. m) counter-clockwise; returns m, or 0 when the edges do not close into one
+// ring.
 __device__ __forceinline__ int ring_of_lines(const Sh &s, int n)
 {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     int *cl = s.ring, *cn = cl + kLines, *cp = cn + kLines, *rk = cp + kLines;
-    float area = 0.0f;
     int m = 0;
 #pragma unroll 1
     for (int i = lane; i < kLines; i += 32) {
@@ -1158,15 +1157,10 @@ __device__ __forceinline__ int ring_of_lines(const Sh &s, int n)
         rk[i] = alive ? r : -1;
         if (alive) {
             cl[r] = i; cn[r] = __float_as_int(p.w); cp[r] = __float_as_int(p.z);
-            // twice the triangle of the edge and the origin, less what rounding can make of it (below
-            // 1e-6 of the edge: the origin lies in the face, so the sum has no cancellation)
-            area += (-s.line[i].z - 2e-6f) * (p.y - p.x);
         }
         m += __popc(b);
     }
     __syncwarp();
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) area += __shfl_xor_sync(full, area, o);
     bool ok = m >= 3 && m <= 32;
     int nxt = -1, prv = -1, k = -1;
     if (ok && lane < m) {
@@ -1187,7 +1181,6 @@ __device__ __forceinline__ int ring_of_lines(const Sh &s, int n)
     } while (cur != 0 && left > 0);
     if (cur != 0 || left != 0) return 0;             // no cycle, or a shorter one
     if (lane < m) s.pe[0][pos] = k;
-    if (lane == 0) s.si[6] = area > 1e-12f ? 1 : 2;
     __syncwarp();
     return m;
 }
@@ -1435,7 +1428,13 @@ __device__ __forceinline__ bool fast_face(const MarchArgs &a, int N, const Sh &s
         AM_PHASE(a, 4, tq0, tq1);
         const int m = s.si[0];
         if (m == 0) return false;
-        // ---- a5: every row at every vertex
+        // ---- a5: every row at every vertex; the area flag s.si[6] (1: clear of the smallest kept area, 2:
+        //      FP64 decides) by the last warp, which has the fewest rows
+        if (wid == kNW - 1) {
+            const float4 *v = reinterpret_cast<const float4 *>(s.vf);
+            const bool clear = area_clear(v[0], v[m / 3], v[2 * m / 3], area_min(a.box_hi));
+            if (lane == 0) s.si[6] = clear ? 1 : 2;
+        }
         float Xm = 1.0f;
         if (M == kDF)
 #pragma unroll 1
