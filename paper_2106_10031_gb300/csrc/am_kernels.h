@@ -10,6 +10,22 @@
 
 namespace am {
 
+// Lets every launch of a kernel take up to the device's dynamic shared memory; cudaErrorInvalidValue when `bytes`
+// is above that.  The attribute belongs to the function, which all contexts of the process launch, so it
+// is never set to one context's size: a later, smaller context would have the launches of an earlier one refused.
+inline cudaError_t allow_smem(const void *kernel, int bytes)
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)fa.sharedSizeBytes;
+    if (bytes > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // candidate rows clipped before the all-row check
 enum { kCandNearest = 0, kCandLearned = 1, kCandNone = 2 };
 

@@ -2219,20 +2219,12 @@ void launch_compose(const MarchArgs &a, int mode, const NetDev *net, const unsig
 cudaError_t prepare_march_kernels(int max_n, int max_w, int *blocks_per_sm)
 {
     const int smem = march_smem_bytes(max_n, max_w);
+    const void *ks[6] = {(const void *)march_persistent_kernel<kFP64>, (const void *)march_persistent_kernel<kDF>,
+                         (const void *)march_range_kernel<kFP64>, (const void *)march_range_kernel<kDF>,
+                         (const void *)compose_kernel<kFP64>, (const void *)compose_kernel<kDF>};
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(march_persistent_kernel<kFP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    if ((e = cudaFuncSetAttribute(march_persistent_kernel<kDF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    if ((e = cudaFuncSetAttribute(march_range_kernel<kFP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    if ((e = cudaFuncSetAttribute(march_range_kernel<kDF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    if ((e = cudaFuncSetAttribute(compose_kernel<kFP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    if ((e = cudaFuncSetAttribute(compose_kernel<kDF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    // shared memory for two resident blocks, the rest of the unified L1 for the weights and
-    // the stack (the driver rounds the carveout to a supported split)
-    const int carve = std::min(100, (int)((2.0 * (smem + 1024) * 100.0) / (228.0 * 1024.0)) + 3);
-    const void *ks[4] = {(const void *)march_persistent_kernel<kFP64>, (const void *)march_persistent_kernel<kDF>,
-                         (const void *)march_range_kernel<kFP64>, (const void *)march_range_kernel<kDF>};
     for (const void *k : ks)
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return e;
+        if ((e = allow_smem(k, smem))) return e;
     int b0 = 0, b1 = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, march_persistent_kernel<kFP64>, kT, smem))) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, march_persistent_kernel<kDF>, kT, smem))) return e;
@@ -2243,12 +2235,24 @@ cudaError_t prepare_march_kernels(int max_n, int max_w, int *blocks_per_sm)
 void launch_march(const MarchArgs &a, int mode, bool persistent, int grid, cudaStream_t st)
 {
     const int smem = march_smem_bytes(a.max_n, a.max_w);
+    // shared memory for two resident blocks, the rest of the unified L1 for the weights and the stack (the
+    // driver rounds the carveout to a supported split); said per launch, as it depends on the context
+    cudaLaunchAttribute carve{};
+    carve.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    carve.val.sharedMemCarveout = (unsigned)std::min(100, (int)((2.0 * (smem + 1024) * 100.0) / (228.0 * 1024.0)) + 3);
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3(kT);
+    c.dynamicSmemBytes = (size_t)smem;
+    c.stream = st;
+    c.attrs = &carve;
+    c.numAttrs = 1;
     if (persistent) {
-        if (mode == kDF) march_persistent_kernel<kDF><<<grid, kT, smem, st>>>(a);
-        else march_persistent_kernel<kFP64><<<grid, kT, smem, st>>>(a);
+        if (mode == kDF) cudaLaunchKernelEx(&c, march_persistent_kernel<kDF>, a);
+        else cudaLaunchKernelEx(&c, march_persistent_kernel<kFP64>, a);
     } else {
-        if (mode == kDF) march_range_kernel<kDF><<<grid, kT, smem, st>>>(a);
-        else march_range_kernel<kFP64><<<grid, kT, smem, st>>>(a);
+        if (mode == kDF) cudaLaunchKernelEx(&c, march_range_kernel<kDF>, a);
+        else cudaLaunchKernelEx(&c, march_range_kernel<kFP64>, a);
     }
 }
 

@@ -719,15 +719,14 @@ __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(PairArgs a)
 
 cudaError_t prepare_seed_kernels(int max_n, int max_w)
 {
-    const int bytes = seed_smem_bytes(max_n, max_w);
-    cudaError_t e = cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(trace_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sample_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    const int dbytes = df_seed_smem_bytes(max_n, max_w);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sample_eval_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dbytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(seed_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dbytes);
+    const int bytes = seed_smem_bytes(max_n, max_w), dbytes = df_seed_smem_bytes(max_n, max_w);
+    const void *plain[3] = {(const void *)seed_kernel, (const void *)trace_kernel, (const void *)sample_eval_kernel};
+    const void *df[2] = {(const void *)sample_eval_df_kernel, (const void *)seed_df_kernel};
+    cudaError_t e = cudaSuccess;
+    for (const void *k : plain)
+        if (e == cudaSuccess) e = allow_smem(k, bytes);
+    for (const void *k : df)
+        if (e == cudaSuccess) e = allow_smem(k, dbytes);
     return e;
 }
 
