@@ -192,7 +192,9 @@ typedef struct {
     int64_t kernel_launches;  /* all kernel launches of the library since the last am_reset */
     int64_t close_calls;      /* mixed precision: sign tests re-evaluated in FP64 */
     int64_t fixups;           /* faces whose candidate polygon the all-row check corrected */
-    int64_t cuts;             /* half-plane cuts applied to face polygons (candidates + corrections) */
+    int64_t cuts;             /* half-plane cuts applied to face polygons one by one (candidates +
+                                 corrections); a face closed in one pass over its candidate lines
+                                 (FP64 and mixed marches with the nearest candidates) takes none */
     int64_t phase_cycles[10]; /* SM cycles summed over cells per phase (compose, candidate lines,
                                  candidate sort, edge intervals, ring and FP64 vertices, check, emit,
                                  push, waiting for work, sequential clip); only filled by a build with

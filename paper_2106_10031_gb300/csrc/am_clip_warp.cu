@@ -826,9 +826,9 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
             kk[2] = -1;
             __syncwarp();
         }
-        n_cuts += ncut;
         if (!fallback && a.chk && m <= kChkMaxV) {
             // the dense check runs on the tensor cores (check_tc); the finish pass emits the cell
+            n_cuts += ncut;
             unsigned long long q = 0;
             if (lane == 0) q = atomicAdd(a.chk_count, 1ull);
             q = __shfl_sync(FULL, q, 0);
@@ -859,6 +859,7 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
         n_solved += 1;
         if (!emit) n_empty += 1;
         if (rounds) n_fix += 1;
+        n_cuts += ncut;
         n_close += (unsigned)close;                      // per lane, summed at the end
         if (!emit) continue;
 #pragma unroll 1

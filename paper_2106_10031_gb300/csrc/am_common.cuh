@@ -46,7 +46,7 @@ enum {
     kCloseCalls = 8 * kCtrStride,   // mixed precision: sign tests re-evaluated in FP64
     kFixups = 9 * kCtrStride,       // faces whose candidate polygon the full check corrected
     kPhase0 = 10 * kCtrStride,      // 10 per-phase cycle counters (timing builds only)
-    kCuts = 20 * kCtrStride,        // half-plane cuts applied to candidate polygons (clip work)
+    kCuts = 20 * kCtrStride,        // half-plane cuts applied to face polygons one by one
     kWarpFallback = 21 * kCtrStride,  // cells the warp clip handed to the block kernel
     kNumCounters = 22 * kCtrStride
 };

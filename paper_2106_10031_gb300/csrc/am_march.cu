@@ -170,7 +170,7 @@ struct Sh {
     int *nid;               // and its net
     unsigned long long *blk;   // per-block statistics, flushed once when the block exits:
                                // 0 solved, 1 empty, 2 degenerate, 3 fixups, 4 refined, 5 close calls,
-                               // 6 cuts
+                               // 6 cuts of the sequential clip
 };
 
 extern __shared__ __align__(16) unsigned char march_smem[];
@@ -1418,10 +1418,7 @@ __device__ __forceinline__ bool fast_face(const MarchArgs &a, int N, const Sh &s
         if (wid == 0) {
             const int m = ring_of_lines(s, n);
             const bool ok = m > 0 && ring_vertices<M>(a.ar, s, m, N);
-            if (lane == 0) {
-                s.si[0] = ok ? m : 0;
-                s.blk[6] += (unsigned long long)m;
-            }
+            if (lane == 0) s.si[0] = ok ? m : 0;
         }
         __syncthreads();
         AM_TICK(tq1);

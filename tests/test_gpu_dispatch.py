@@ -68,3 +68,22 @@ def test_march_edges(oracle_mod, make, box, precision, schedule):
     r = parity.compare(ref, mesh, mlp.N, rtol=1e-5 if precision == "mixed" else 1e-9)
     assert st["faces"] == r["faces"] > 0 and mesh.n_open_faces == ref.open_faces()
     assert mesh.n_open_faces > 0                         # each of these surfaces meets the box
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_one_pass_faces_count_no_cuts(precision):
+    # the counter holds cuts applied one by one: several a face without candidates, none for the faces that
+    # close in one pass (all but the few that the sequential clip takes)
+    import paper_2106_10031_gb300 as am
+    mlp = geometric_init([33, 31], 5, 0.05, recenter=True)
+    per_cell = {}
+    with am.Mesher(max_cells=1 << 16, max_neurons=64, max_width=33) as m:
+        nid = m.load_mlp(mlp)
+        for candidates in ("none", "nearest"):
+            m.reset()
+            m.seed(nid, np.zeros((1, 3)), X_RAY, 2.0)
+            m.march(precision=precision, candidates=candidates)
+            st = m.stats()
+            per_cell[candidates] = st["cuts"] / st["cells"]
+    assert per_cell["none"] >= 3.0                       # a closed polygon takes three cuts or more
+    assert per_cell["nearest"] < 0.5
