@@ -20,16 +20,17 @@ namespace am {
 
 // ---- products of BF16 operands on the FP32 pipes
 //
-// Every element is one chain of fused multiply-adds over k in ascending order from zero, so a result does
-// not depend on the tile, the launch or the device's load (a split of k, or the tensor cores' own order,
-// would move the BF16 roundings between the layers).  What bounds a training step of this MLP (batch 1024,
-// 15 -> 256 -> 256 -> 2048: 1.8 G multiply-adds, 46 us at the FP32 peak) is keeping the FP32 pipes fed
-// along chains of up to 2048 k: slices of 32 k are staged in shared memory as FP32, the next two slices'
-// loads in flight while one is multiplied, the operands of the next k read while those of one are
-// multiplied, each thread keeps a TM x TN block of sums, and the products that wait for the same input
-// share one launch, with their bias, activation, loss or backward step as the epilogue.  A step takes
-// 291 us; 933 with a 64 x 64 kernel per product (4 loads per 8 multiply-adds, strided global reads), its
-// element-wise kernels and a copy of the loss to the host per step.
+// Every element of a product is one chain of fused multiply-adds over k in ascending order from zero, so it
+// does not depend on the tile, the launch or the device's load (a split of k, or the tensor cores' own order,
+// would move the BF16 roundings between the layers).  The loss and the bias gradients are sums of partial sums
+// whose number follows the tile, so with another batch their last bits may differ; runs repeat bit for bit.
+// What bounds a training step of this MLP (batch 1024, 15 -> 256 -> 256 -> 2048: 1.8 G multiply-adds, 46 us at
+// the FP32 peak) is keeping the FP32 pipes fed along chains of up to 2048 k: slices of 32 k are staged in
+// shared memory as FP32, the next two slices' loads in flight while one is multiplied, the operands of the
+// next k read while those of one are multiplied, each thread keeps a TM x TN block of sums, and the products
+// that wait for the same input share one launch, with their bias, activation, loss or backward step as the
+// epilogue.  A step takes 291 us; 933 with a 64 x 64 kernel per product (4 loads per 8 multiply-adds, strided
+// global reads), its element-wise kernels and a copy of the loss to the host per step.
 
 constexpr int kGK = 32;     // K slice
 constexpr int kLossSteps = 4096;     // losses kept on the device between copies
@@ -57,7 +58,8 @@ struct GemmJobs {
     int n;
 };
 
-// db[c] = sum over rows of C[r, c]: 32 columns per block, the rows in groups combined in shared memory
+// db[c] = sum over rows of C[r, c]: 32 columns per block, the rows in T / 32 groups (8 or 4, with the launch's
+// tile) combined in shared memory
 template <int T>
 __device__ __forceinline__ void colsum_block(const GemmJob &g, int tile, float *sh)
 {
@@ -254,7 +256,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) gemm_jobs_kernel(const 
 struct JobList {
     GemmJobs q{};
     void add(const GemmJob &g) { q.j[q.n++] = g; }
-    void run(cudaStream_t st)
+    // launches them; returns the number of tiles (of a product with the loss: its partial sums)
+    int run(cudaStream_t st)
     {
         // 64 x 64 tiles (3 shared-memory wavefronts per 16 multiply-adds of a warp) when they fill the
         // chip twice, else 32 x 32 (four times as many, of half the threads): the logits of 1024 samples
@@ -278,6 +281,7 @@ struct JobList {
             gemm_jobs_kernel<32, 32, 2, 4><<<t, 128, 0, st>>>(q);
         }
         q = GemmJobs{};
+        return t;
     }
 };
 
@@ -490,8 +494,8 @@ void proposal_sync_copies(ProposalDev &p, cudaStream_t st)
 
 // Forward pass over B samples (B <= max_batch).  Activations: buf0 a1, buf1 a2 (FP32, for the backward
 // pass); bbuf0 x, bbuf1 h1, bbuf2 h2 (BF16).  Without labels the logits go to buf2; with labels Y the loss's
-// partial sums to loss_parts and dz to buf3 (FP32) and bbuf3 (BF16).
-static void forward(ProposalDev &p, const float *X, const float *Y, int B, cudaStream_t st)
+// partial sums to loss_parts and dz to buf3 (FP32) and bbuf3 (BF16).  Returns the number of partial sums.
+static int forward(ProposalDev &p, const float *X, const float *Y, int B, cudaStream_t st)
 {
     const int H = p.hidden, I = p.n_in, O = p.n_out;
     const __nv_bfloat16 *W1 = p.wb + p.off[0], *W2 = p.wb + p.off[2], *W3 = p.wb + p.off[4];
@@ -515,14 +519,7 @@ static void forward(ProposalDev &p, const float *X, const float *Y, int B, cudaS
     g.scale = 1.0f / (float)((int64_t)B * O);
     g.loss_parts = p.loss_parts;
     q.add(g);
-    q.run(st);
-}
-
-// partial sums of the loss that a forward pass over B samples leaves (as JobList::run tiles it)
-static int loss_tiles(const ProposalDev &p, int B)
-{
-    auto t = [&](int d) { return ((B + d - 1) / d) * ((p.n_out + d - 1) / d); };
-    return t(64) >= 2 * 152 ? t(64) : t(32);
+    return q.run(st);
 }
 
 // Gradients (into p.g) over B samples, after forward with labels.  da2: buf5, bbuf4; da1: buf6, bbuf5.
@@ -577,9 +574,9 @@ cudaError_t proposal_forward(ProposalDev &p, const float *X, int n, float *Z, cu
 cudaError_t proposal_grad(ProposalDev &p, const float *X, const float *Y, int n, float *loss, cudaStream_t st)
 {
     if (n > p.max_batch) return cudaErrorInvalidValue;
-    forward(p, X, Y, n, st);
+    const int parts = forward(p, X, Y, n, st);
     backward(p, n, st);
-    loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, loss_tiles(p, n), (double)n * p.n_out, p.losses);
+    loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, parts, (double)n * p.n_out, p.losses);
     cudaError_t e = cudaMemcpyAsync(loss, p.losses, sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e) return e;
     return cudaStreamSynchronize(st);
@@ -593,7 +590,7 @@ cudaError_t proposal_train(ProposalDev &p, const float *X, const float *Y, int64
     int done = 0;                                // losses copied out; the device keeps up to kLossSteps
     for (int it = 0; it < steps; ++it) {
         if (cursor + batch > n) cursor = 0;
-        forward(p, X + cursor * p.n_in, Y + cursor * p.n_out, batch, st);
+        const int parts = forward(p, X + cursor * p.n_in, Y + cursor * p.n_out, batch, st);
         backward(p, batch, st);
         cursor += batch;
         p.step += 1;
@@ -603,7 +600,7 @@ cudaError_t proposal_train(ProposalDev &p, const float *X, const float *Y, int64
         cudaError_t e = cudaGetLastError();
         if (e) return e;
         if (!losses) continue;
-        loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, loss_tiles(p, batch), (double)batch * p.n_out, p.losses + (it - done));
+        loss_kernel<<<1, 256, 0, st>>>(p.loss_parts, parts, (double)batch * p.n_out, p.losses + (it - done));
         if (it + 1 - done == kLossSteps || it + 1 == steps) {
             e = cudaMemcpyAsync(losses + done, p.losses, sizeof(float) * (it + 1 - done), cudaMemcpyDeviceToHost, st);
             if (e) return e;

@@ -323,3 +323,18 @@ def test_learned_256x8_trained_on_other_nets(oracle_mod, am, torch):
     assert stats["learned"]["ms_march"] < stats["plain"]["ms_march"]
     assert stats["learned"]["ms_proposal"] > 0.0            # scored on the tensor cores, per batch
     parity.compare_sampled(oracle_mod, oracle_mod.OracleNet(mlp), meshes["learned"], mlp.N, 16, 1e-9, 1.5)
+
+
+def test_loss_counts_every_tile_once(am, torch):
+    """With all parameters zero every logit is 0 and every element's loss log 2, so the mean is log 2 whatever
+    the labels (FP32 sums of at most 64 x 64 equal terms, each rounding at most 2^-24 of the sum: 2^-17 in
+    all); a partial sum left out, read twice or left over from a larger batch would move it by the inverse
+    of the number of tiles.  Batches on both sides of the change of tile, the largest first."""
+    O = 2049
+    with am.Mesher(max_cells=1024, max_neurons=64, max_width=32) as m:
+        m.proposal_init(8, 32, O, max_batch=1024, seed=5)
+        m.proposal_set_params(np.zeros_like(m.proposal_params()))
+        for B in (1024, 577, 576, 64, 33, 1):            # 528, 330, 297 of the large tiles, then small ones
+            X, Y = _rand_xy(B, 8, O, 13)
+            loss, _ = m.proposal_grad(torch.as_tensor(X, device="cuda"), torch.as_tensor(Y, device="cuda"))
+            assert abs(loss - np.log(2.0)) <= 2 ** -17, (B, loss)
