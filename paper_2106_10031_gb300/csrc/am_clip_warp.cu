@@ -9,9 +9,11 @@
 //   candidates : each lane keeps the two rows nearest to the point the cell was entered through
 //                among the rows it scans, and with learned candidates also the row the proposal
 //                scores highest among them (the proposal extends the nearest set);
-//   clip       : a square about the box section, in FP32 coordinates of the face plane, is cut by the
-//                lines of those 64 (96) candidates, nearest cutting line first, then every vertex
-//                is solved in FP64 from its two planes (Eq. 11);
+//   clip       : a square about that point, in FP32 coordinates of the face plane, is cut by the lines of
+//                those 64 (96) candidates, nearest cutting line first, then every vertex is solved
+//                in FP64 from its two planes (Eq. 11).  The square need not contain the box's
+//                section (a seed may lie outside the box): a cell with an edge of it left goes to
+//                the block kernel;
 //   check      : every row at every vertex with a certified FP32 bound; the rows it does not clear
 //                (the edges' own among them) one by one, close calls in FP64; violated rows join
 //                the edges as the lines of another round;
@@ -37,39 +39,33 @@ constexpr int kWMaxKw = 128;      // key words (N <= 8190)
 constexpr int kWMaxFix = 8;       // check / fix-up rounds
 constexpr float kWU = 5.9604645e-8f;   // 2^-24
 
+// a warp of the finish pass (after the dense check on the tensor cores)
 struct WarpSh {
     double pv[2][kWPoly][3];      // FP64 polygon
-    float pf[2][kWPoly][3];       // FP32 polygon of the candidate pass
+    float mid[kWPoly][3];         // the edges' midpoints, for the pushes
     int pe[2][kWPoly];            // edge planes (edge i: vertex i -> i + 1)
     float4 vf[kWPoly];            // FP32 vertices (x, y, z) and the vertex term of the check's bound (w)
     int2 ve[kWPoly];              // the planes of the two edges at each vertex
     float dvb[kWPoly];            // bound on each FP64 vertex's error
-    float sq[4][4];               // the initial square's rows (planes N + 6 .. N + 9)
     int viol[kWViol];
     double aF[4];
-    float aFhi[4];
-    int nviol, flag;
+    int nviol;
     unsigned key[2 * kWMaxKw];    // the cell's key as 32-bit words (pushes copy it)
 };
 
 int warp_smem_bytes() { return kWW * (int)sizeof(WarpSh); }
 
-// the rows of one cell: N rows in memory, the 6 box rows and the 4 square rows analytic
+// the rows of one cell: N rows in memory, the 6 box rows analytic
 struct WRows {
     const float4 *p;              // [hi, lo] per row
     int N;
     float box, box_lo;            // the box as an FP32 pair: box rows' offsets -box (hi), -box_lo (lo)
-    const WarpSh *S;
     __device__ __forceinline__ float4 hi(int k) const
     {
         if (k < N) return __ldg(p + k);
-        if (k < N + kBoxPlanes) {
-            const int i = k - N;
-            const float sg = (i & 1) ? -1.0f : 1.0f;
-            return make_float4((i >> 1) == 0 ? sg : 0.0f, (i >> 1) == 1 ? sg : 0.0f, (i >> 1) == 2 ? sg : 0.0f, -box);
-        }
-        const float *q = S->sq[k - N - kBoxPlanes];
-        return make_float4(q[0], q[1], q[2], q[3]);
+        const int i = k - N;
+        const float sg = (i & 1) ? -1.0f : 1.0f;
+        return make_float4((i >> 1) == 0 ? sg : 0.0f, (i >> 1) == 1 ? sg : 0.0f, (i >> 1) == 2 ? sg : 0.0f, -box);
     }
     __device__ __forceinline__ void f64(int k, double *r) const
     {
@@ -80,7 +76,7 @@ struct WRows {
             r[2] = (double)h.z + (double)l.z; r[3] = (double)h.w + (double)l.w;
         } else {
             r[0] = h.x; r[1] = h.y; r[2] = h.z;
-            r[3] = k < N + kBoxPlanes ? (double)h.w - (double)box_lo : (double)h.w;
+            r[3] = (double)h.w - (double)box_lo;
         }
     }
 };
@@ -182,60 +178,21 @@ __device__ __forceinline__ void wload_key(WarpSh &S, const Arena &ar, int64_t ce
     }
 }
 
-// The cell's rows view, key and face plane a_F in the warp's shared memory, then (lane 0) the
-// face plane's FP32 frame and the square about the box section: the initial polygon in buffer 0
-// (planes N + 6 .. N + 9).  Returns its vertex count, 0 when a_F has no normal.
-__device__ int wcell_setup(const MarchArgs &a, WarpSh &S, int64_t cell, int N, WRows &rv)
+// The cell's rows view, and its key and face plane a_F in the warp's shared memory
+__device__ void wcell_setup(const MarchArgs &a, WarpSh &S, int64_t cell, int N, WRows &rv)
 {
     const int lane = threadIdx.x & 31;
     rv.p = reinterpret_cast<const float4 *>(a.rows_in) + (cell - a.begin) * 2 * (int64_t)(N + 1);
     rv.N = N;
     rv.box = a.box_hi;
     rv.box_lo = a.box_lo;
-    rv.S = &S;
     wload_key(S, a.ar, cell);
     if (lane < 4) {
         const float h = reinterpret_cast<const float *>(rv.p + N)[lane];
         const float l = reinterpret_cast<const float *>(rv.p + 2 * N + 1)[lane];   // lo block: N + 1 + N
         S.aF[lane] = (double)h + (double)l;
-        S.aFhi[lane] = h;
     }
     __syncwarp();
-    int m = 0;
-    if (lane == 0) {
-        const float F[4] = {(float)S.aF[0], (float)S.aF[1], (float)S.aF[2], (float)S.aF[3]};
-        const float nn = F[0] * F[0] + F[1] * F[1] + F[2] * F[2];
-        if (nn > 0.0f && isfinite(nn)) {
-            const float inn = 1.0f / nn;
-            const float p0[3] = {-F[3] * F[0] * inn, -F[3] * F[1] * inn, -F[3] * F[2] * inn};
-            const float inv = rsqrtf(nn);
-            const float n[3] = {F[0] * inv, F[1] * inv, F[2] * inv};
-            const float ax = fabsf(n[0]), ay = fabsf(n[1]), az = fabsf(n[2]);
-            const int ei = (ax <= ay && ax <= az) ? 0 : (ay <= az ? 1 : 2);
-            const float e0 = ei == 0 ? 1.0f : 0.0f, e1 = ei == 1 ? 1.0f : 0.0f, e2 = ei == 2 ? 1.0f : 0.0f;
-            float u[3] = {n[1] * e2 - n[2] * e1, n[2] * e0 - n[0] * e2, n[0] * e1 - n[1] * e0};
-            const float un = rsqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-            u[0] *= un; u[1] *= un; u[2] *= un;
-            const float w[3] = {n[1] * u[2] - n[2] * u[1], n[2] * u[0] - n[0] * u[2], n[0] * u[1] - n[1] * u[0]};
-            const float sz = 1.05f * 1.7320508f * (float)a.box;
-            const float d[4][3] = {{-w[0], -w[1], -w[2]}, {u[0], u[1], u[2]}, {w[0], w[1], w[2]}, {-u[0], -u[1], -u[2]}};
-            const float cu[4] = {-1.0f, 1.0f, 1.0f, -1.0f}, cw[4] = {-1.0f, -1.0f, 1.0f, 1.0f};
-            for (int i = 0; i < 4; ++i) {
-                S.sq[i][0] = d[i][0]; S.sq[i][1] = d[i][1]; S.sq[i][2] = d[i][2];
-                S.sq[i][3] = -(d[i][0] * p0[0] + d[i][1] * p0[1] + d[i][2] * p0[2]) - sz;
-                for (int c = 0; c < 3; ++c) {
-                    const float x = p0[c] + sz * (cu[i] * u[c] + cw[i] * w[c]);
-                    S.pv[0][i][c] = (double)x;
-                    S.pf[0][i][c] = x;
-                }
-                S.pe[0][i] = N + kBoxPlanes + i;
-            }
-            m = 4;
-        }
-    }
-    m = __shfl_sync(0xffffffffu, m, 0);
-    __syncwarp();
-    return m;
 }
 
 // A close call of the FP32 test: row k at the FP64 vertex v6 from the exact pair, against the
@@ -353,15 +310,13 @@ __device__ bool wcheck(const MarchArgs &a, WarpSh &S, const WRows &rv, int N, in
     return fallback;
 }
 
-// a6 emit, a7 march for a solved cell: the face record (empty when it has fewer than 3 vertices,
-// a square edge, or no area), then one push per neuron edge; returns whether a face was written
+// a6 emit, a7 march for a solved cell: the face record (empty when it has fewer than 3 vertices or no
+// area), then one push per neuron edge; returns whether a face was written
 __device__ bool wemit(const MarchArgs &a, WarpSh &S, int64_t cell, int net_id, int N, int m, int buf)
 {
     const int lane = threadIdx.x & 31;
     const Arena &ar = a.ar;
     int emit = m >= 3 ? m : 0;
-    for (int i = 0; i < m; ++i)
-        if (S.pe[buf][i] >= N + kBoxPlanes) emit = 0;     // a square edge: the plane misses the box
     if (emit) {
         const double *p0 = S.pv[buf][0];
         double nx = 0.0, ny = 0.0, nz = 0.0;
@@ -387,9 +342,8 @@ __device__ bool wemit(const MarchArgs &a, WarpSh &S, int64_t cell, int net_id, i
             v[0] = S.pv[buf][i][0]; v[1] = S.pv[buf][i][1]; v[2] = S.pv[buf][i][2];
         }
         const unsigned long long h = __ldcg(ar.hash + cell);
-        // the entry point of each neighbour (the midpoint of the shared edge), one edge per lane,
-        // kept in the FP32 polygon's buffer (buf ^ 1 is free: the face is in buf)
-        float (*mid)[3] = S.pf[buf ^ 1];
+        // the entry point of each neighbour (the midpoint of the shared edge), one edge per lane
+        float (*mid)[3] = S.mid;
         for (int i = lane; i < m; i += 32) {
             const double *p = S.pv[buf][i], *q = S.pv[buf][i + 1 == m ? 0 : i + 1];
             mid[i][0] = (float)(0.5 * (p[0] + q[0]));
@@ -673,7 +627,7 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
         unsigned ncut = 0;
         float vx = 0.0f, vy = 0.0f;
         while (!fallback) {
-            // ---- the candidate clip (FP32, in the plane): a square about the box section, then the nearest
+            // ---- the candidate clip (FP32, in the plane): a square about the entry point, then the nearest
             //      cutting line first; a line that holds on the polygon holds on every smaller one and retires
             float cA[3], cB[3], cC[3];
             bool live[3];
@@ -684,7 +638,9 @@ __global__ void __launch_bounds__(kWW * 32, AM_CLIP_MIN_BLOCKS) clip_warp_kernel
                 cA[j] = L.x; cB[j] = L.y; cC[j] = L.z;
                 live[j] = kk[j] >= 0;
             }
-            const float sz = 2.1f * 1.7320508f * box;    // the entry point lies in the box
+            // reaches past the box from any point in it; from a point outside, an edge of the square may
+            // remain, which the block kernel takes
+            const float sz = 2.1f * 1.7320508f * box;
             vx = (lane == 1 || lane == 2) ? sz : -sz;
             vy = lane >= 2 ? sz : -sz;
             float eA = lane == 1 ? 1.0f : (lane == 3 ? -1.0f : 0.0f), eB = lane == 0 ? -1.0f : (lane == 2 ? 1.0f : 0.0f), eC = -sz;
@@ -907,12 +863,12 @@ __global__ void __launch_bounds__(kWW * 32) clip_warp_finish_kernel(MarchArgs a)
             wload_key(S, ar, cell);
         } else {
             WRows rv;
-            fallback = wcell_setup(a, S, cell, N, rv) == 0;   // key, a_F and the square's rows
+            wcell_setup(a, S, cell, N, rv);
             for (int i = lane; i < m; i += 32) {
                 S.pe[0][i] = R.pe[i];
             }
             __syncwarp();
-            if (!fallback) fallback = !wfinal(S, m, 0, rv);     // the same FP64 vertices and their bounds
+            fallback = !wfinal(S, m, 0, rv);                    // the same FP64 vertices and their bounds
             if (!fallback) fallback = wcheck(a, S, rv, N, m, buf, rounds, ncut, cell_close);
         }
         if (fallback) {
