@@ -123,7 +123,8 @@ int march_smem_bytes(int max_n, int max_w)
     return lay_total(max_n);
 }
 
-// The proposal's scores use the compose scratch: 64 features + 2 hidden layers + 2 kT partials.
+// The proposal's scores use the scratch region below the net's record: 64 features + 2 hidden layers + 2 kT
+// partial sums.
 int proposal_max_hidden() { return (kOHot / 4 - 64 - 2 * kT) / 2; }
 
 // The tensor-core compose keeps one layer's B fragments (16 bytes per lane per 16 input rows)
@@ -1074,7 +1075,8 @@ __device__ void proposal_scores(const MarchArgs &a, const NetDev &net, int64_t c
 {
     const ProposalView &P = a.prop;
     const int tid = threadIdx.x, H = P.hidden, O = P.n_out, I = P.n_in;
-    float *x = s.partf;            // the compose partial sums are free here
+    // the start of the scratch region, up to the net's record at kOHot, which stays (proposal_max_hidden)
+    float *x = s.partf;
     float *h1 = x + 64, *h2 = h1 + H, *part = h2 + H;
     if (tid == 0) {
         x[0] = __ldcg(a.ar.entry_pt + cell * 3);

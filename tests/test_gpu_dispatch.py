@@ -87,3 +87,46 @@ def test_one_pass_faces_count_no_cuts(precision):
             per_cell[candidates] = st["cuts"] / st["cells"]
     assert per_cell["none"] >= 3.0                       # a closed polygon takes three cuts or more
     assert per_cell["nearest"] < 0.5
+
+
+def _clip(C, aF):
+    """The polygon {aF [x; 1] = 0, C [x; 1] <= 0}, cut row by row out of a large square (or None)."""
+    n = aF[:3] / np.linalg.norm(aF[:3])
+    u = np.cross(n, np.eye(3)[np.argmin(np.abs(n))])
+    u /= np.linalg.norm(u)
+    w, p0 = np.cross(n, u), -aF[3] / np.linalg.norm(aF[:3]) * n
+    P = [p0 + 5.0 * (a * u + b * w) for a, b in ((-1, -1), (1, -1), (1, 1), (-1, 1))]
+    for c in C:
+        v = [c[:3] @ p + c[3] for p in P]
+        P = [q for i in range(len(P)) for q in
+             ([P[i - 1] + v[i - 1] / (v[i - 1] - v[i]) * (P[i] - P[i - 1])] if (v[i - 1] <= 0) != (v[i] <= 0) else [])
+             + ([P[i]] if v[i] <= 0 else [])]
+        if len(P) < 3:
+            return None
+    return np.array(P)
+
+
+@pytest.mark.parametrize("precision,schedule", [("fp64", "persistent"), ("mixed", "persistent"), ("sliced", "levels")])
+def test_seeds_outside_the_box(oracle_mod, precision, schedule):
+    # rays that meet a sphere of radius about 0.6 in a box of half-width 0.45: 16 of 40 seed points lie
+    # outside the box, 14 of them on cells without a face in it, two on faces that the box cuts.  The
+    # oracle's pivoting starts on the face, so for these two it starts from a point of the cut face.
+    import paper_2106_10031_gb300 as am
+    mlp, box = geometric_init([32, 32, 32, 32], 21, 0.05), 0.45
+    d = np.random.default_rng(3).normal(size=(40, 3))
+    d /= np.linalg.norm(d, axis=1)[:, None]
+    o = np.zeros((40, 3))
+    net, seeds = oracle_mod.OracleNet(mlp), []
+    for key, x in oracle_mod.seed_cells(net, o, d, 2.0):
+        P = [x] if np.abs(x).max() <= box else _clip(*net.cell_rows(oracle_mod.key_to_state(key, mlp.N), box))
+        if P is not None:
+            seeds.append((key, np.mean(P, axis=0)))
+    assert len(seeds) == 26
+    ref = oracle_mod.march(net, seeds, box)
+    with am.Mesher(max_cells=1 << 16, max_neurons=mlp.N, max_width=32) as m:
+        nid = m.load_mlp(mlp)
+        m.seed(nid, o, d, 2.0)
+        m.march(box=box, precision=precision, schedule=schedule)
+        mesh, st = m.get_mesh(nid), m.stats()
+    parity.compare(ref, mesh, mlp.N, rtol=1e-5 if precision == "mixed" else 1e-9)
+    assert st["empty_faces"] > 0
