@@ -103,8 +103,8 @@ HBM_PEAK_GBS = _measured_hbm_peak()
 # committed ncu capture (every clip launch of the first 399,997 cells of the step's march: 15
 # levels), valid while the kernel source is the one captured; the bench scales it to the cells
 # of an average launch
-TRAFFIC_CAPTURE = {"sha256_prefix": "7363cd8a4451845f", "source": "am_clip_warp.cu", "precision": "sliced",
-                   "candidates": "learned", "cells": 399997, "bytes": 24930303488 + 302267648}
+TRAFFIC_CAPTURE = {"sha256_prefix": "9cd919e2aa3c2467", "source": "am_clip_warp.cu", "precision": "sliced",
+                   "candidates": "learned", "cells": 399997, "bytes": 25000930304 + 251316992}
 
 
 def captured_traffic(precision, candidates, cells_per_launch):
